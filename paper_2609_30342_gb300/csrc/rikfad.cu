@@ -144,6 +144,7 @@ struct rikfad_handle_s {
     bool pageable_ok = false;       // the device reads pageable host memory (host page tables)
     int ntensors = 0;
     int grad_bytes = 4;
+    bool ragged = false;            // a matrix has rows that are not 8-aligned
     rikfad_hparams hp{};
     Plan plan;
     int max_blocks = 1;
@@ -384,14 +385,24 @@ cudaError_t launch_pdl(Kern kernel, int nblocks, int nthreads, cudaStream_t s, c
     return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
 
-template <typename GT>
-cudaError_t launch_step(const StepParams &p, bool reuse, bool shadow, int nblocks, cudaStream_t s)
+using StepKernel = void (*)(StepParams);
+
+// The step kernel's instantiation for a handle's matrices.  Full-friction
+// matrices (shadow) have no pending factor, so reuse never applies to them.
+template <typename GT, bool RAGGED>
+StepKernel step_kernel(bool reuse, bool shadow)
 {
-    if (shadow)     // full-friction matrices: reuse never applies (no pending factor)
-        return launch_pdl(rikfad_step_kernel<GT, false, true>, nblocks, kThreads, s, p);
-    if (reuse)
-        return launch_pdl(rikfad_step_kernel<GT, true>, nblocks, kThreads, s, p);
-    return launch_pdl(rikfad_step_kernel<GT, false>, nblocks, kThreads, s, p);
+    if (shadow)
+        return rikfad_step_kernel<GT, false, true, RAGGED>;
+    return reuse ? rikfad_step_kernel<GT, true, false, RAGGED> : rikfad_step_kernel<GT, false, false, RAGGED>;
+}
+
+StepKernel step_kernel(int grad_bytes, bool reuse, bool shadow, bool ragged)
+{
+    if (grad_bytes == 2)
+        return ragged ? step_kernel<__nv_bfloat16, true>(reuse, shadow)
+                      : step_kernel<__nv_bfloat16, false>(reuse, shadow);
+    return ragged ? step_kernel<float, true>(reuse, shadow) : step_kernel<float, false>(reuse, shadow);
 }
 
 template <typename GT>
@@ -638,13 +649,9 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     RK_CUDA(cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev), "cudaDeviceGetAttribute");
     // Persistent grid: as many blocks as can be resident at once.
     int occ_min = 1 << 30;
-    const void *kernels[6] = {(const void *)rikfad_step_kernel<float, true>,
-                              (const void *)rikfad_step_kernel<float, false>,
-                              (const void *)rikfad_step_kernel<__nv_bfloat16, true>,
-                              (const void *)rikfad_step_kernel<__nv_bfloat16, false>,
-                              (const void *)rikfad_step_kernel<float, false, true>,
-                              (const void *)rikfad_step_kernel<__nv_bfloat16, false, true>};
-    for (const void *k : kernels) {
+    const int grad_bytes = grad_dtype == RIKFAD_GRAD_BF16 ? 2 : 4;
+    for (const bool reuse : {true, false}) {        // the instantiations this handle launches
+        const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, has_ragged(shapes, ntensors));
         RK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kThreads, 0),
                 "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         occ_min = std::min(occ_min, occ);
@@ -675,11 +682,12 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     h->device = dev;
     h->pageable_ok = pageable != 0;
     h->ntensors = ntensors;
-    h->grad_bytes = grad_dtype == RIKFAD_GRAD_BF16 ? 2 : 4;
+    h->grad_bytes = grad_bytes;
     h->hp = *hp;
     h->shapes.assign(shapes, shapes + ntensors);
     h->max_blocks = sms * occ_min;
     h->shadow = shadow;
+    h->ragged = has_ragged(shapes, ntensors);
     why = build_plan(shapes, ntensors, h->grad_bytes, h->max_blocks, h->plan, shadow);
     if (!why.empty()) {
         delete h;
@@ -899,11 +907,9 @@ RIKFAD_API int rikfad_step(rikfad_handle h, double step, float *const *x, const 
                 launch_sweep<float>(a, sp, reuse, h->sweep_blocks, s);
             RK_CUDA(cudaGetLastError(), "launch rikfad_sweep_kernel");
         } else {
-            if (h->grad_bytes == 2)
-                RK_CUDA(launch_step<__nv_bfloat16>(a, reuse, h->shadow, h->plan.nblocks, s),
-                        "launch rikfad_step_kernel");
-            else
-                RK_CUDA(launch_step<float>(a, reuse, h->shadow, h->plan.nblocks, s), "launch rikfad_step_kernel");
+            RK_CUDA(launch_pdl(step_kernel(h->grad_bytes, reuse, h->shadow, h->ragged), h->plan.nblocks,
+                               kThreads, s, a),
+                    "launch rikfad_step_kernel");
         }
     }
     if (ev)

@@ -267,8 +267,24 @@ __global__ void __launch_bounds__(kThreads) rikfad_canonical_kernel(CanonParams 
                     }
                 }
             } else {
-                for (int j = lane; j < pd.width; j += 32)
-                    D[base + j] = (S[base + j] * exp2f(a_prev * Cs[j])) * c.damp_prev;
+                // Rows at any element address: 256 columns' loads before the
+                // first in-place store (one load in flight per lane ran at a
+                // fraction of the bandwidth, as in matrix_piece_ragged).
+                constexpr int kU = 8;
+#pragma unroll 1
+                for (int j0 = lane; j0 < pd.width; j0 += 32 * kU) {
+                    float v[kU];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u)
+                        if (j0 + 32 * u < pd.width)
+                            v[u] = __ldcs(S + base + j0 + 32 * u);
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const int j = j0 + 32 * u;
+                        if (j < pd.width)
+                            __stcs(D + base + j, (v[u] * exp2f(a_prev * Cs[j])) * c.damp_prev);
+                    }
+                }
             }
         }
         __syncthreads();

@@ -148,7 +148,7 @@ template <> struct Grad8<__nv_bfloat16> {
 __device__ __forceinline__ float grad_at(const float *g, int64_t i) { return __ldcs(g + i); }
 __device__ __forceinline__ float grad_at(const __nv_bfloat16 *g, int64_t i)
 {
-    return __bfloat162float(g[i]);
+    return __bfloat162float(__ushort_as_bfloat16(__ldcs(reinterpret_cast<const unsigned short *>(g + i))));
 }
 
 __device__ __forceinline__ void load8(const float *p, float (&v)[8])
@@ -283,15 +283,26 @@ __device__ __forceinline__ void matrix_piece_vec(const StepParams &a, const Piec
     }
 }
 
-// ----------------------------------------------- matrix piece, scalar
-// For matrices whose rows are not 8-aligned (cols % 8 != 0).
-
-template <typename GT, bool REUSE, bool ACCUM = true>
-__device__ __forceinline__ void matrix_piece_scalar(const StepParams &a, const PieceDev &pc,
+// ----------------------------------------------- matrix piece, ragged
+// For matrices whose rows are not 8-aligned (cols % 8 != 0): rows start at any
+// element address, so lanes take single elements; a load instruction of a
+// warp covers consecutive elements of a row.
+//
+// Bound by the bytes in flight: each lane issues its U loads of every array
+// before any arithmetic (U = 8: 256 elements of each array per warp, as on the
+// 8-wide path).  RPW rows per warp as there, so that a narrow panel fills the
+// warp too: each of the RPW lane groups takes its own row.  Measured on a
+// 10007 x 3001 matrix with fp32 gradients (600 MB a step, whole step): one load
+// of each array in flight per lane 281 us, U = 4 144, U = 8 121 and, with
+// streaming hints, 115 (5.2 TB/s); U = 16 was no faster (122 without hints).
+template <typename GT, bool REUSE, bool ACCUM = true, int RPW = 1, int U = 8>
+__device__ __forceinline__ void matrix_piece_ragged(const StepParams &a, const PieceDev &pc,
                                                     const TensorDev &td, const PanelDev &pd,
                                                     const float *Cs, float *red, float inv)
 {
+    constexpr int kRowLanes = 32 / RPW;                 // lanes per row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rl = lane & (kRowLanes - 1), half = lane / kRowLanes;   // lane group = row
     const int64_t n = td.cols;
     const int w = pd.width;
     float *X = a.xptr[pc.tensor];
@@ -299,30 +310,55 @@ __device__ __forceinline__ void matrix_piece_scalar(const StepParams &a, const P
     float *P = a.pptr[pc.tensor];
     const float *R = a.fac + td.fac_off;
     float *rowpart = a.rowpart + td.rowpart_off + (int64_t)(pc.panel - td.panel0) * td.rows;
-    float *myred = red + warp * kPanelMax;
+    float *myred = red + warp * kPanelMax + half * (kPanelMax / RPW);
 
-    for (int64_t row = pc.begin + warp; row < pc.end; row += kWarps) {
-        const float rhat = R[row] * inv;
+    for (int64_t r0 = pc.begin + RPW * warp; r0 < pc.end; r0 += RPW * kWarps) {
+        const int64_t row = r0 + half;
+        const bool live = RPW == 1 || row < pc.end;     // ragged piece: trailing lane groups idle
+        const float rhat = live ? R[row] * inv : 0.f;
         const float a_cur = a.ex_cur * rhat;
         const float a_prev = REUSE ? a_cur : a.ex_prev * rhat;
-        const int64_t base = row * n + pd.col0;
+        const int64_t base = row * n + pd.col0 + rl;
+        float *xr = X + base, *pr = P + base;
+        const GT *gr = G + base;
+        const int wl = live ? w : 0;
         float racc = 0.f;
-        for (int c = lane; c < w; c += 32) {
-            const float e_cur = exp2f(a_cur * Cs[c]);
-            const float e_prev = REUSE ? e_cur : exp2f(a_prev * Cs[c]);
-            float x = X[base + c];
-            const float p1 = matrix_element(x, P[base + c], grad_at(G, base + c), e_cur, e_prev, a);
-            X[base + c] = x;
-            P[base + c] = p1;
-            const float q = p1 * p1;
-            racc += q;
-            if (ACCUM)
-                myred[c] += q;
-            else
-                myred[c] = q;
+#pragma unroll 1
+        for (int c0 = rl; c0 < wl; c0 += kRowLanes * U) {
+            float x[U], p[U], g[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (c0 + kRowLanes * u < w) {
+                    g[u] = grad_at(gr, kRowLanes * u);
+                    x[u] = __ldcs(xr + kRowLanes * u);
+                    p[u] = __ldcs(pr + kRowLanes * u);
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int c = c0 + kRowLanes * u;
+                if (c < w) {
+                    const float cv = Cs[c];
+                    const float e_cur = exp2f(a_cur * cv);
+                    const float e_prev = REUSE ? e_cur : exp2f(a_prev * cv);
+                    const float p1 = matrix_element(x[u], p[u], g[u], e_cur, e_prev, a);
+                    __stcs(xr + kRowLanes * u, x[u]);
+                    __stcs(pr + kRowLanes * u, p1);
+                    const float q = p1 * p1;
+                    racc += q;
+                    if (ACCUM)
+                        myred[c] += q;
+                    else
+                        myred[c] = q;
+                }
+            }
+            xr += kRowLanes * U;
+            pr += kRowLanes * U;
+            gr += kRowLanes * U;
         }
-        racc = warp_sum(racc);
-        if (lane == 0)
+#pragma unroll
+        for (int o = kRowLanes / 2; o > 0; o >>= 1)
+            racc += __shfl_xor_sync(0xffffffffu, racc, o);
+        if (live && rl == 0)
             rowpart[row] = racc;
     }
 }
@@ -402,7 +438,7 @@ __device__ __forceinline__ float full_element(float &x, float &p, float &xi, flo
     return p1 * p1;
 }
 
-template <typename GT>
+template <typename GT, bool RAGGED>
 __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const PieceDev &pc,
                                                   const TensorDev &td, const PanelDev &pd,
                                                   float *red)
@@ -419,7 +455,7 @@ __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const Pie
     for (int64_t row = pc.begin + warp; row < pc.end; row += kWarps) {
         const int64_t base = row * n + pd.col0;
         float racc = 0.f;
-        if (td.vec) {
+        if (!RAGGED || td.vec) {
 #pragma unroll 1
             for (int ch = 0; ch < pd.nch; ++ch) {
                 const int c = ch * kChunk + lane * 8;
@@ -448,14 +484,33 @@ __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const Pie
                 }
             }
         } else {
-            for (int c = lane; c < w; c += 32) {
-                float x = X[base + c], p = P[base + c], xi = XI[base + c];
-                const float q = full_element(x, p, xi, grad_at(G, base + c), a);
-                X[base + c] = x;
-                P[base + c] = p;
-                XI[base + c] = xi;
-                racc += q;
-                myred[c] += q;
+            // Rows at any element address: 256 columns' loads before any
+            // arithmetic, as matrix_piece_ragged.
+            constexpr int kU = 8;
+#pragma unroll 1
+            for (int c0 = lane; c0 < w; c0 += 32 * kU) {
+                float x[kU], p[kU], xi[kU], g[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (c0 + 32 * u < w) {
+                        const int64_t i = base + c0 + 32 * u;
+                        g[u] = grad_at(G, i);
+                        x[u] = __ldcs(X + i);
+                        p[u] = __ldcs(P + i);
+                        xi[u] = __ldcs(XI + i);
+                    }
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int c = c0 + 32 * u;
+                    if (c < w) {
+                        const float q = full_element(x[u], p[u], xi[u], g[u], a);
+                        __stcs(X + base + c, x[u]);
+                        __stcs(P + base + c, p[u]);
+                        __stcs(XI + base + c, xi[u]);
+                        racc += q;
+                        myred[c] += q;
+                    }
+                }
             }
         }
         racc = warp_sum(racc);
@@ -471,9 +526,11 @@ __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const Pie
 #define RIKFAD_STEP_MIN_BLOCKS 2
 #endif
 
-// SHADOW: the instantiation for handles whose matrices keep element-wise
-// friction with shadow factors (the R-iKFAD instantiation carries no code for
-// it).
+// SHADOW: the instantiation for handles whose matrices all keep element-wise
+// friction with shadow factors (the R-iKFAD instantiations carry no code for
+// it, nor it any for them).  RAGGED: the instantiation for handles with a
+// matrix whose rows are not 8-aligned; the paths of such matrices take more
+// registers than the 8-wide ones, so other handles do not carry them.
 // out[c] = the piece's column sums: warp wi's lane group h holds its share at
 // red[wi * kPanelMax + h * kPanelMax / RPW + c]; added warp by warp, groups in
 // order.
@@ -491,17 +548,21 @@ __device__ __forceinline__ void column_partials(const float *red, float *out, in
     }
 }
 
-// Rows per warp for an 8-wide panel (matrix_piece_vec RPW): a panel that is
-// not a whole number of 256-column chunks takes 4 rows per warp up to 64
-// columns and 2 up to kPanelMax / 2 columns; every other panel takes 1.
-__device__ __forceinline__ int rows_per_warp(int w)
+// Rows per warp (RPW of matrix_piece_vec and matrix_piece_ragged).  An 8-wide
+// panel that is not a whole number of 256-column chunks takes 4 rows per warp
+// up to 64 columns and 2 up to kPanelMax / 2 columns; every other one takes 1.
+// A ragged panel takes as many as leave every lane its 8 elements: 4 up to 64
+// columns, 2 up to 128.
+__device__ __forceinline__ int rows_per_warp(bool vec, int w)
 {
+    if (!vec)
+        return w <= kChunk / 4 ? 4 : w <= kChunk / 2 ? 2 : 1;
     if (w % kChunk == 0 || w > kPanelMax / 2)
         return 1;
     return w <= kChunk / 4 ? 4 : 2;
 }
 
-template <typename GT, bool REUSE, bool SHADOW = false>
+template <typename GT, bool REUSE, bool SHADOW = false, bool RAGGED = false>
 __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_kernel(StepParams a)
 {
     __shared__ __align__(16) float Cs[kPanelMax];
@@ -542,21 +603,27 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
             red[i] = 0.f;
         const float inv = inv_denominator(row_total(a.spart, td), a.eps);
         __syncthreads();
-        if (SHADOW && td.full) {
-            matrix_piece_full<GT>(a, pc, td, pd, red);
-        } else if (td.vec && rows_per_warp(w) == 4) {
-            matrix_piece_vec<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
-        } else if (td.vec && rows_per_warp(w) == 2) {
-            matrix_piece_vec<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
-        } else if (td.vec) {
-            matrix_piece_vec<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
+        const int rpw = SHADOW ? 1 : rows_per_warp(!RAGGED || td.vec, w);
+        if (SHADOW) {
+            matrix_piece_full<GT, RAGGED>(a, pc, td, pd, red);
+        } else if (!RAGGED || td.vec) {
+            if (rpw == 4)
+                matrix_piece_vec<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
+            else if (rpw == 2)
+                matrix_piece_vec<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
+            else
+                matrix_piece_vec<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
         } else {
-            matrix_piece_scalar<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
+            if (rpw == 4)
+                matrix_piece_ragged<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
+            else if (rpw == 2)
+                matrix_piece_ragged<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
+            else
+                matrix_piece_ragged<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
         }
         __syncthreads();
         // Column partial sums of this piece, warps (and their lane groups) added in order.
         float *out = a.colpart + pc.colpart_off;
-        const int rpw = td.vec && !(SHADOW && td.full) ? rows_per_warp(w) : 1;
         if (rpw == 1)
             column_partials<1>(red, out, w);
         else if (rpw == 2)

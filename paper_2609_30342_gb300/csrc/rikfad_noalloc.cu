@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS)
     if (na.vec)
         matrix_piece_vec<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
     else
-        matrix_piece_scalar<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
+        matrix_piece_ragged<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
     __syncthreads();
     for (int c = tid; c < w; c += kThreads) {
         float t = 0.f;

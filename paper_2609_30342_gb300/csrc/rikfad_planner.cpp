@@ -53,6 +53,14 @@ std::string check_shapes(const rikfad_shape *shapes, int ntensors)
     return "";
 }
 
+bool has_ragged(const rikfad_shape *shapes, int ntensors)
+{
+    for (int t = 0; t < ntensors; ++t)
+        if (shapes[t].rows > 0 && shapes[t].cols % 8 != 0)
+            return true;
+    return false;
+}
+
 std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes, int max_blocks,
                        Plan &plan, bool full_matrices)
 {
@@ -129,7 +137,8 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
                 if (td.rows > 0) {
                     const int64_t b = pd.width * (full_matrices ? vector_elem_bytes(grad_bytes)
                                                                 : matrix_elem_bytes(grad_bytes));
-                    units.push_back({kMatrixRows, t, (int32_t)p.panels.size(), td.rows, b + kRowCost, 1, b});
+                    const int64_t c = td.vec ? b : b * kRaggedNum / kRaggedDen;
+                    units.push_back({kMatrixRows, t, (int32_t)p.panels.size(), td.rows, c + kRowCost, 1, b});
                 }
                 p.panels.push_back(pd);
             }

@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_SWEEP_MIN_BLOCKS)
         if (td.vec)
             matrix_piece_vec<GT, REUSE, false>(a, pc, td, pd, Cs, red, inv);
         else
-            matrix_piece_scalar<GT, REUSE, false>(a, pc, td, pd, Cs, red, inv);
+            matrix_piece_ragged<GT, REUSE, false, 1, 1>(a, pc, td, pd, Cs, red, inv);
         __syncthreads();
         // Column partial of the unit: its rows' squares, warps in order.
         const int nrows = (int)(un.end - un.begin);

@@ -1,0 +1,82 @@
+"""Matrices whose rows are not 8-aligned (cols % 8 != 0), on the GPU against
+the oracle: widths at the edges of the kernels' tiles (32-element load
+instructions, 8 per lane; 4, 2 and 1 rows per warp up to 64, 128 and more
+columns; panels of 1024), odd row counts, and buffers that start at any
+element address."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import HParams
+from paper_2609_30342_gb300 import build as pkg_build
+from paper_2609_30342_gb300 import workloads
+
+from gpu_helpers import DeviceRun, Tracked
+from test_gpu_diagnostics import HP as SHADOW_HP, ShadowRef, _compare, _gpu_state
+
+pytestmark = pytest.mark.gpu
+
+WIDTHS = [1, 31, 33, 63, 65, 127, 129, 255, 257, 511, 1023, 1025, 2051]
+SHAPES = [(r, w) for w, r in zip(WIDTHS, [70, 9, 33, 31, 1, 17, 66, 8, 23, 5, 16, 3, 2])] + [(40, 64), (13, 0)]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    pkg_build.build()
+    yield
+
+
+def _off_by_one(run):
+    """Move the ragged matrices' buffers one element on: 4-byte (fp32) and
+    2-byte (bf16) aligned bases."""
+    for lst in (run.x, run.p, run.g, run.out):
+        for t, (m, n) in enumerate(run.shapes):
+            if n % 8:
+                flat = torch.empty(m * n + 1, dtype=lst[t].dtype, device="cuda")
+                v = flat[1:].view(m, n)
+                v.copy_(lst[t])
+                lst[t] = v
+    run.ptrs = run.opt.pack(run.x, run.g, run.p)
+
+
+@pytest.mark.parametrize("shift", [False, True])
+@pytest.mark.parametrize("grad_bf16", [True, False])
+def test_ragged_steps_match_oracle(grad_bf16, shift):
+    """Constant and changing step sizes (one and two exponentials per element),
+    from the GPU's own state at every step: 1e-5, per-element rounding bound
+    beyond it.  Summation depths: a lane's <= 8 columns a pass, 5 butterfly
+    levels and 3 panels; a warp's rows, 8 warps x 4 groups and the slots; 64 covers
+    both."""
+    hp = HParams(alpha=0.3, mu=1e-3, gamma=0.05, eps_stab=1e-8)
+    inp = workloads.ModelInputs(SHAPES, seed=61, g_std=1e-2, grad_bf16=grad_bf16)
+    run = DeviceRun(SHAPES, hp, grad_bf16, inp.X, inp.P)
+    if shift:
+        _off_by_one(run)
+    for k, h in enumerate((0.1, 0.1, 0.05)):
+        seeded = Tracked.from_gpu(run)
+        g = inp.grads(k)
+        run.set_grads(g)
+        run.step(h)
+        seeded.step(g, h, hp, run.factors())
+        seeded.check(run, 1e-5, "step%d" % (k + 1))
+    # in place: the same bits as out of place
+    want = run.canonical_P()
+    run.opt.materialize(run.p)
+    torch.cuda.synchronize()
+    for p, w in zip(run.p, want):
+        assert np.array_equal(p.double().cpu().numpy(), w)
+    run.close()
+
+
+@pytest.mark.parametrize("grad_bf16", [True, False])
+def test_ragged_shadow_steps_match_oracle(grad_bf16):
+    inp = workloads.ModelInputs(SHAPES, seed=62, g_std=1e-2, grad_bf16=grad_bf16)
+    run = DeviceRun(SHAPES, SHADOW_HP, grad_bf16, inp.X, inp.P, method="ikfad_shadow")
+    for k, h in enumerate((0.1, 0.05)):
+        seeded = ShadowRef(SHAPES, *_gpu_state(run))
+        g = inp.grads(k)
+        run.set_grads(g)
+        run.step(h)
+        seeded.step(g, h)
+        _compare(run, seeded, 1e-5, "reseeded step%d " % (k + 1))
+    run.close()
