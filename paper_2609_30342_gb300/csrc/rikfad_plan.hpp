@@ -37,8 +37,8 @@ constexpr int64_t kRowCost = 256;
 // A ragged row (cols % 8 != 0, moved in single elements) costs kRaggedNum /
 // kRaggedDen of its bytes: in a list of 8-wide matrices the blocks that hold
 // one ragged matrix finish last otherwise.  GPT2-S and one 1001 x 769 matrix
-// step in 412 us without the factor, 365 with 5/4 and 363 with 3/2 (the list alone in 355).
-constexpr int64_t kRaggedNum = 3, kRaggedDen = 2;
+// step in 412 us without the factor, 365 with it (363 with 3/2; the list alone 355).
+constexpr int64_t kRaggedNum = 5, kRaggedDen = 4;
 
 enum PieceKind : int32_t { kMatrixRows = 0, kElements = 1 };
 enum FinKind : int32_t { kFinRows = 0, kFinCols = 1 };
