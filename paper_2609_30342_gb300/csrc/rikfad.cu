@@ -175,10 +175,11 @@ struct rikfad_handle_s {
 
     // full iKFAD with shadow R-iKFAD factors (friction diagnostics)
     bool shadow = false;
-    float *d_diag_u = nullptr, *d_diag_v = nullptr, *d_diag_w = nullptr, *d_diag_wpart = nullptr;
-    double *d_diag_norms = nullptr, *d_diag_upart = nullptr, *d_diag_wsq = nullptr;
+    float *d_diag_v = nullptr, *d_diag_wpart = nullptr;
+    double *d_diag_norms = nullptr, *d_diag_upart = nullptr, *d_diag_v2part = nullptr;
     DiagState *d_diag_state = nullptr;
-    DiagState *h_diag_state = nullptr;   // pinned
+    DiagState *h_diag_state = nullptr;      // mapped page-locked host memory
+    DiagState *h_diag_state_dev = nullptr;  // its device address
 
     // in-order ("sweep") schedule, allocated only when selected
     bool sweep = false;
@@ -340,8 +341,8 @@ void release(rikfad_handle h)
     for (void *p : {(void *)h->d_tensors, (void *)h->d_panels, (void *)h->d_pieces, (void *)h->d_block_piece,
                     (void *)h->d_slot_off, (void *)h->d_fin, (void *)h->d_fac, (void *)h->d_rowpart,
                     (void *)h->d_colpart, (void *)h->d_spart, (void *)h->d_den, (void *)h->d_guard,
-                    (void *)h->d_checks, (void *)h->d_diag_u, (void *)h->d_diag_v, (void *)h->d_diag_w,
-                    (void *)h->d_diag_wpart, (void *)h->d_diag_norms, (void *)h->d_diag_upart, (void *)h->d_diag_wsq,
+                    (void *)h->d_checks, (void *)h->d_diag_v, (void *)h->d_diag_wpart,
+                    (void *)h->d_diag_norms, (void *)h->d_diag_upart, (void *)h->d_diag_v2part,
                     (void *)h->d_diag_state, (void *)h->d_units, (void *)h->d_nodes,
                     (void *)h->d_trees, (void *)h->d_partials, (void *)h->d_counts, (void *)h->d_fetch})
         rk_free(p);
@@ -370,12 +371,12 @@ int64_t numel(const TensorDev &td) { return td.cols == 0 ? td.rows : td.rows * t
 // its predecessor in the stream finishes; it waits (griddepcontrol.wait)
 // before touching any data.
 template <typename Kern, typename Arg>
-cudaError_t launch_pdl(Kern kernel, int nblocks, int nthreads, cudaStream_t s, const Arg &arg)
+cudaError_t launch_pdl(Kern kernel, int nblocks, int nthreads, cudaStream_t s, const Arg &arg, size_t smem = 0)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nblocks);
     cfg.blockDim = dim3((unsigned)nthreads);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -739,26 +740,24 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
         if (!rc) rc = alloc_zero((float **)&h->d_fetch, 4, ws);
     }
     if (!rc && shadow) {
-        int64_t max_m = 1, max_n = 1, max_parts = 1;
+        int64_t max_n = 1, max_wpart = 1;
         for (const TensorDev &td : p.tensors)
-            if (td.cols > 0) {
-                max_m = std::max(max_m, td.rows);
+            if (td.cols > 0 && td.rows > 0) {
                 max_n = std::max(max_n, td.cols);
-                max_parts = std::max<int64_t>(max_parts, (td.rows + diag_rows_per_group(td.rows) - 1) /
-                                                             diag_rows_per_group(td.rows));
+                max_wpart = std::max(max_wpart, diag_row_blocks(td.rows, td.cols) * td.cols);
             }
-        rc = alloc_zero(&h->d_diag_u, max_m, ws);
-        if (!rc) rc = alloc_zero(&h->d_diag_v, max_n, ws);
-        if (!rc) rc = alloc_zero(&h->d_diag_w, max_n, ws);
-        if (!rc) rc = alloc_zero(&h->d_diag_wpart, max_parts * max_n, ws);
-        if (!rc) rc = alloc_zero((float **)&h->d_diag_norms, 4 * ((max_m + kWarps - 1) / kWarps), ws);
-        if (!rc) rc = alloc_zero((float **)&h->d_diag_upart, 2 * ((max_m + kWarps - 1) / kWarps), ws);
-        if (!rc) rc = alloc_zero((float **)&h->d_diag_wsq, 2 * ((max_n + 31) / 32), ws);
+        rc = alloc_zero(&h->d_diag_v, max_n, ws);
+        if (!rc) rc = alloc_zero(&h->d_diag_wpart, max_wpart, ws);
+        if (!rc) rc = alloc_zero((float **)&h->d_diag_norms, 4 * kDiagMaxBlocks, ws);
+        if (!rc) rc = alloc_zero((float **)&h->d_diag_upart, 2 * kDiagMaxBlocks, ws);
+        if (!rc) rc = alloc_zero((float **)&h->d_diag_v2part, 4 * kDiagMaxColBlocks, ws);
         if (!rc) rc = alloc_zero((float **)&h->d_diag_state, (int64_t)(sizeof(DiagState) / sizeof(float)), ws);
         if (!rc) {
-            cudaError_t e = rk_malloc_host((void **)&h->h_diag_state, sizeof(DiagState), cudaHostAllocDefault);
+            cudaError_t e = rk_malloc_host((void **)&h->h_diag_state, sizeof(DiagState), cudaHostAllocMapped);
             if (e != cudaSuccess)
-                rc = alloc_fail(e, "cudaHostAlloc of the diagnostic state read-back");
+                rc = alloc_fail(e, "cudaHostAlloc of the diagnostic state record");
+            else if ((e = cudaHostGetDevicePointer((void **)&h->h_diag_state_dev, h->h_diag_state, 0)) != cudaSuccess)
+                rc = cuda_fail(e, "cudaHostGetDevicePointer");
         }
     }
     if (!rc) rc = ptrtable_init(h->step_ptrs, 3 * ntensors, ws);
@@ -1224,86 +1223,47 @@ RIKFAD_API int rikfad_friction_diagnostics(rikfad_handle h, int t, int max_iters
     if (m == 0)
         return RIKFAD_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    const float *xi = h->d_fac + td.xi_off;
-    const float *R = h->d_fac + td.fac_off;
-    const float *C = h->d_fac + td.fac_off + m;
-    // 1^T R exactly as the step kernels form it, then inv, the start vector
-    // (C normalised) and a cleared iteration state, all on the device.
-    DenParams d{h->d_tensors, h->d_spart, h->d_den, h->ntensors, bounds(h)};
-    rikfad_denominators_kernel<<<(h->ntensors + kWarps - 1) / kWarps, kThreads, 0, s>>>(d);
-    rikfad_diag_setup_kernel<<<1, kDiagFinThreads, 0, s>>>(h->d_den + t, (float)h->hp.eps_stab, C, n,
-                                                           h->d_diag_v, h->d_diag_state);
-    // ||xi||^2 and ||xi - xi~||^2
-    const int nb_rows = (int)((m + kWarps - 1) / kWarps);
-    rikfad_diag_norms_kernel<<<nb_rows, kThreads, 0, s>>>(xi, m, n, R, C, h->d_diag_state, h->d_diag_norms);
-    RK_CUDA(cudaGetLastError(), "launch diagnostic set-up kernels");
-    // sigma_1 by power iteration on xi^T xi, starting from C (the shadow
-    // column factor, close to the top right singular vector).  A batch of
-    // kBatch iterations (four kernels each) and the read-back of the state
-    // record are captured once into a CUDA graph, which is replayed until
-    // the iteration is done; after convergence the remaining kernels of a
-    // batch return at once.  One graph launch replaces 32 kernel launches.
-    const int nb_t = (int)((m + diag_rows_per_group(m) - 1) / diag_rows_per_group(m));
-    const dim3 grid_t((unsigned)nb_t, (unsigned)((n + kThreads - 1) / kThreads));
-    const int nb_c = (int)((n + 31) / 32);
-    constexpr int kBatch = 8;
-    DiagState &st = *h->h_diag_state;
-    cudaStream_t cs = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    auto cleanup = [&]() {
-        if (exec)
-            cudaGraphExecDestroy(exec);
-        if (graph)
-            cudaGraphDestroy(graph);
-        if (cs)
-            cudaStreamDestroy(cs);
-    };
-    cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-    if (e == cudaSuccess)
-        e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        for (int b = 0; b < kBatch; ++b) {
-            rikfad_diag_matvec_kernel<<<nb_rows, kThreads, 0, cs>>>(xi, m, n, h->d_diag_v, h->d_diag_u,
-                                                                    h->d_diag_upart, h->d_diag_state);
-            rikfad_diag_matvec_t_kernel<<<grid_t, kThreads, 0, cs>>>(xi, m, n, h->d_diag_u, h->d_diag_wpart,
-                                                                     h->d_diag_state);
-            rikfad_diag_colsum_kernel<<<nb_c, kDiagFinThreads, 0, cs>>>(h->d_diag_wpart, nb_t, n, h->d_diag_w,
-                                                                 h->d_diag_wsq, h->d_diag_state);
-            rikfad_diag_iterate_kernel<<<1, kDiagFinThreads, 0, cs>>>(h->d_diag_w, n, h->d_diag_wsq, nb_c,
-                                                                     h->d_diag_upart, nb_rows, h->d_diag_v,
-                                                                     h->d_diag_state, tol, max_iters);
+    DiagParams d{};
+    d.xi = h->d_fac + td.xi_off;
+    d.R = h->d_fac + td.fac_off;
+    d.C = h->d_fac + td.fac_off + m;
+    d.spart = h->d_spart;
+    d.td = td;
+    d.eps = (float)h->hp.eps_stab;
+    d.nblk = (int)diag_row_blocks(m, n);
+    d.wpr = diag_warps_per_row(m);
+    d.ncb = diag_col_blocks(n);
+    d.cpb = diag_cols_per_block(n);
+    d.max_iters = max_iters;
+    d.tol = tol;
+    d.v = h->d_diag_v;
+    d.wpart = h->d_diag_wpart;
+    d.upart = h->d_diag_upart;
+    d.npart = h->d_diag_norms;
+    d.v2part = h->d_diag_v2part;
+    d.st = h->d_diag_state;
+    d.host = h->h_diag_state_dev;
+    // Iterations are enqueued kDiagIters at a time; after convergence the
+    // kernels left in the queue return at once.
+    const bool vec = n % 4 == 0 && n <= kDiagStageCols;
+    const size_t smem = n <= kDiagStageCols ? (size_t)((n + 3) / 4 * 8) * sizeof(float) : 0;
+    const DiagState &st = *h->h_diag_state;
+    RK_CUDA(cudaMemsetAsync(h->d_diag_state, 0, sizeof(DiagState), s), "cudaMemsetAsync");
+    for (int it = 0; it < max_iters;) {
+        const int64_t stop = std::min<int64_t>(max_iters, (int64_t)it + kDiagIters);
+        for (; it < stop; ++it) {
+            d.parity = it & 1;
+            d.last = it + 1 == stop;
+            auto rows = it == 0 ? (vec ? rikfad_diag_rows_kernel<true, true> : rikfad_diag_rows_kernel<true, false>)
+                                : (vec ? rikfad_diag_rows_kernel<false, true> : rikfad_diag_rows_kernel<false, false>);
+            RK_CUDA(launch_pdl(rows, d.nblk, kThreads, s, d, smem), "launch rikfad_diag_rows_kernel");
+            RK_CUDA(launch_pdl(rikfad_diag_cols_kernel, d.ncb, kThreads, s, d), "launch rikfad_diag_cols_kernel");
         }
-        cudaMemcpyAsync(h->h_diag_state, h->d_diag_state, sizeof(DiagState), cudaMemcpyDeviceToHost, cs);
-        e = cudaStreamEndCapture(cs, &graph);
-    }
-    if (e == cudaSuccess)
-        e = cudaGraphInstantiate(&exec, graph, 0);
-    if (e != cudaSuccess) {
-        cleanup();
-        return cuda_fail(e, "capture of the power iteration");
-    }
-    for (int enqueued = 0; enqueued < max_iters; enqueued += kBatch) {
-        e = cudaGraphLaunch(exec, s);
-        if (e == cudaSuccess)
-            e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) {
-            cleanup();
-            return cuda_fail(e, "power iteration");
-        }
+        RK_CUDA(cudaStreamSynchronize(s), "power iteration");
         if (st.done)
             break;
     }
-    cleanup();
-    std::vector<double> parts(2 * (size_t)nb_rows);
-    RK_CUDA(cudaMemcpyAsync(parts.data(), h->d_diag_norms, sizeof(double) * parts.size(), cudaMemcpyDeviceToHost, s),
-            "cudaMemcpyAsync");
-    RK_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
-    double f2 = 0.0, e2 = 0.0;
-    for (int b = 0; b < nb_rows; ++b) {
-        f2 += parts[2 * b];
-        e2 += parts[2 * b + 1];
-    }
+    const double f2 = st.f2, e2 = st.e2;
     const double sigma2 = st.sigma2;
     const int it = st.it;
     const double sigma1 = std::sqrt(sigma2);

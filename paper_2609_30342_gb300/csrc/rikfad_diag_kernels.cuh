@@ -3,43 +3,105 @@
 // from the full element-wise friction xi of the same trajectory, against the
 // best rank-1 approximation (Eckart-Young: relative error
 // sqrt(1 - sigma_1^2 / ||xi||_F^2)), and the stable rank ||xi||_F^2 /
-// sigma_1^2 (the comparison of the paper's Section 4.4).  sigma_1 comes from
-// power iteration on xi^T xi: two matrix-vector passes over xi per iteration
-// (HBM-bound GEMVs; there is no dense contraction to put on tensor cores).
-// The iteration runs on the device: the transposed product writes one
-// partial per row group and column, a column kernel adds them, a one-block
-// kernel normalises the iterate, forms the Rayleigh quotient and tests
-// convergence, and every kernel of the loop returns at once after
-// convergence, so the host enqueues iterations in batches and reads one small
-// state record per batch.  Every reduction runs in a fixed order.  Float64
-// is slow on this GPU: per element the kernels compute in float32, and
-// float64 only adds partial sums (per row, per column block, per block).
+// sigma_1^2 (the comparison of the paper's Section 4.4).
+//
+// sigma_1 comes from power iteration on xi^T xi, on the device, two kernels an
+// iteration chained by programmatic dependent launch: the row kernel reads xi
+// once from memory (u = xi v, then this block's share of xi^T u from the rows
+// just read, still in L1 or L2), the column kernel adds the blocks' shares,
+// forms the next iterate and tests convergence.  The first row kernel also
+// takes the norms ||xi||^2 and ||xi - xi~||^2 from the same read.
+//
+// The iterate's length does not matter: sigma^2 = ||xi v||^2 / ||v||^2 is formed
+// with the length of the float32 iterate itself, so no kernel waits for a norm
+// over all columns, and a rounding of v enters the quotient at second order
+// only.  What would enter at first order, the rounding of u = xi v, is kept
+// below 1e-13 by compensated dot products (Ogita, Rump and Oishi, "Accurate sum
+// and dot product", 2005, algorithm Dot2) in float32, about ten times the rate
+// of float64 here.  So the quotient settles as soon as the iterate has
+// converged: 2 to 4 iterations for GPT2-S layers, where a quotient from plain
+// float32 sums wandered by ~1e-9 for 10 to 200 until two in a row agreed to
+// 1e-10.
+//
+// Every reduction runs in a fixed order; float64 only adds per-row and
+// per-block partial sums.  Bound by launch and L2 latency for a layer's 2 to 10
+// MB, by the one read of xi for larger matrices.  Measured on GB300, six calls
+// for the layers of a GPT2-S block: 3800 to 7400 us (by seed) with four kernels an
+// iteration in a captured graph and the plain quotient, 354 us so.
 #pragma once
+#include <algorithm>
+
 #include "rikfad_kernels.cuh"
 
 namespace rikfad {
 
-constexpr int kDiagFinThreads = 1024;    // threads of the one-block kernels
-constexpr int kDiagBatch = 8;            // loads a thread issues before consuming them
-constexpr int kDiagMaxRowGroups = 512;   // row groups of the transposed product (partials per column)
+constexpr int kDiagMaxBlocks = 456;      // row blocks: 3 per SM of a GB300
+constexpr int kDiagStageCols = 4096;     // widest xi whose iterate and sums are staged in shared memory
+constexpr int kDiagMaxColBlocks = 512;   // column blocks (each adds all of their sums of v^2)
+constexpr int64_t kDiagMaxPartials = 1 << 24;   // floats of row-block partials (more only at 32 rows a block)
+constexpr int kDiagIters = 4;            // iterations enqueued before the host looks
 
-// Rows per block of the transposed product: at least 32, with at most
-// kDiagMaxRowGroups row groups (partials per column for the column kernel).
-inline __host__ __device__ int64_t diag_rows_per_group(int64_t m)
-{
-    const int64_t r = (m + kDiagMaxRowGroups - 1) / kDiagMaxRowGroups;
-    return r < 32 ? 32 : r;
-}
-
-// State of one power iteration, in device memory (read back by the host).
+// State of one power iteration, in device memory; the record the host reads
+// is a copy in mapped host memory.
 struct DiagState {
-    double sigma2;     // Rayleigh quotient ||xi v||^2 of the current unit iterate
-    double w2;         // ||xi^T xi v||^2
+    double sigma2;     // ||xi v||^2 / ||v||^2 of the current iterate
+    double f2;         // ||xi||^2
+    double e2;         // ||xi - xi~||^2
     int32_t it;        // iterations done
     int32_t done;      // converged, or max_iters reached, or xi^T xi v = 0
-    float inv;         // 1 / (1^T R + eps_stab) of the shadow factors (0 if zero)
-    int32_t pad_;
 };
+
+struct DiagParams {
+    const float *xi;           // m x n, row-major, 16-byte aligned
+    const float *R, *C;
+    const float *spart;
+    TensorDev td;
+    float eps;
+    int nblk;                  // blocks of the row kernel
+    int wpr;                   // warps per row: 1, 2, 4 or 8
+    int ncb;                   // blocks of the column kernel
+    int64_t cpb;               // columns of each, a multiple of 32
+    int parity;                // which half of v2part holds ||v||^2 of this iteration
+    int last;                  // 1: write the host's record even if not done
+    int max_iters;
+    double tol;
+    float *v;                  // iterate (written by the column kernel)
+    float *wpart;              // nblk x n
+    double *upart;             // nblk: sums of u_i^2
+    double *npart;             // 2 x nblk: sums of xi^2 and (xi - xi~)^2
+    double *v2part;            // 2 x ncb: sums of v_j^2
+    DiagState *st;
+    DiagState *host;           // mapped host memory
+};
+
+// Warps per row: as many as give the row kernel a block per SM of a GB300.
+inline int diag_warps_per_row(int64_t m)
+{
+    int wpr = 1;
+    while (wpr < kWarps && m * wpr < 152 * kWarps)
+        wpr *= 2;
+    return wpr;
+}
+
+// Blocks of the row kernel.  Their partials stay within kDiagMaxPartials where
+// that leaves at least a block per 32 rows.
+inline int64_t diag_row_blocks(int64_t m, int64_t n)
+{
+    const int64_t rows = kWarps / diag_warps_per_row(m);
+    const int64_t blocks = std::min<int64_t>(kDiagMaxBlocks, (m + rows - 1) / rows);
+    return std::min(blocks, std::max(kDiagMaxPartials / n, (m + 31) / 32));
+}
+
+// Columns per block of the column kernel, a multiple of 32, and its blocks.
+inline int64_t diag_cols_per_block(int64_t n)
+{
+    return (n + 32 * kDiagMaxColBlocks - 1) / (32 * kDiagMaxColBlocks) * 32;
+}
+
+inline int diag_col_blocks(int64_t n)
+{
+    return (int)((n + diag_cols_per_block(n) - 1) / diag_cols_per_block(n));
+}
 
 __device__ __forceinline__ double warp_sum_f64(double v)
 {
@@ -49,266 +111,359 @@ __device__ __forceinline__ double warp_sum_f64(double v)
     return v;
 }
 
-// Block-wide sum of one double per thread, threads in a fixed tree order;
-// the result is returned to every thread.  Float64 arithmetic is slow on
-// this GPU, so only warp 0 combines the warp sums and the total is passed on
-// through shared memory (scratch holds NT / 32 + 1 doubles).
-template <int NT>
-__device__ __forceinline__ double block_sum_f64(double v, double *scratch)
+// s + e += a b, with the rounding errors of the product and of the sum in e.
+__device__ __forceinline__ void dot2(float &s, float &e, float a, float b)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    v = warp_sum_f64(v);
-    __syncthreads();
-    if (lane == 0)
-        scratch[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        double t = lane < NT / 32 ? scratch[lane] : 0.0;
-        t = warp_sum_f64(t);
-        if (lane == 0)
-            scratch[NT / 32] = t;
-    }
-    __syncthreads();
-    return scratch[NT / 32];
+    const float p = __fmul_rn(a, b);
+    const float pe = __fmaf_rn(a, b, -p);
+    const float t = __fadd_rn(s, p);
+    const float z = __fsub_rn(t, s);
+    e += __fadd_rn(pe, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z)));
+    s = t;
 }
 
-// Start of a diagnostic: inv from 1^T R (den, as the step kernels form it),
-// the unit start vector v = C / ||C|| (1/sqrt(n) per entry if C = 0), and a
-// cleared state.  One block.
-__global__ void __launch_bounds__(kDiagFinThreads) rikfad_diag_setup_kernel(const float *den, float eps,
-                                                                           const float *C, int64_t n,
-                                                                           float *v, DiagState *st)
+// (s, e) += (s2, e2)
+__device__ __forceinline__ void add2(float &s, float &e, float s2, float e2)
 {
-    __shared__ double scratch[kDiagFinThreads / 32 + 1];
-    __shared__ double s_scale;
-    double a = 0.0;
-    for (int64_t j = threadIdx.x; j < n; j += kDiagFinThreads)
-        a += (double)C[j] * (double)C[j];
-    const double c2 = block_sum_f64<kDiagFinThreads>(a, scratch);
-    // One float64 square root and division for the block (float64 is slow on
-    // this GPU), then a multiply per entry.
-    if (threadIdx.x == 0)
-        s_scale = c2 > 0.0 ? 1.0 / sqrt(c2) : 0.0;
-    __syncthreads();
-    const double sc = s_scale;
-    const float uniform = (float)(1.0 / sqrt((double)n));
-    for (int64_t j = threadIdx.x; j < n; j += kDiagFinThreads)
-        v[j] = sc > 0.0 ? (float)((double)C[j] * sc) : uniform;
-    if (threadIdx.x == 0) {
-        const float d = *den + eps;
-        st->inv = d == 0.f ? 0.f : 1.f / d;
-        st->sigma2 = 0.0;
-        st->w2 = 0.0;
-        st->it = 0;
-        st->done = 0;
-    }
+    const float t = __fadd_rn(s, s2);
+    const float z = __fsub_rn(t, s);
+    e = __fadd_rn(__fadd_rn(e, e2), __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(s2, z)));
+    s = t;
 }
 
-// Per block of 8 rows (one per warp): sum of xi^2 and of (xi - xi~)^2,
-// written to part[2 * block] and part[2 * block + 1].  A row is added in
-// float32 (xi - xi~ is the difference of two floats, exact where they are
-// within a factor two of each other): each lane its elements, then the 32
-// lanes by a butterfly; the rows and the blocks are added in float64.
-__global__ void __launch_bounds__(kThreads) rikfad_diag_norms_kernel(const float *xi, int64_t m, int64_t n,
-                                                                     const float *R, const float *C,
-                                                                     const DiagState *st, double *part)
+// Row kernel.  A block takes a contiguous range of rows, kWarps / wpr at a
+// time: wpr warps a row for u_i (columns interleaved between them), then every
+// thread its own columns for the block's share of xi^T u.  FIRST: the iterate
+// is C, scaled to at most unit length (all ones over sqrt(n) if C = 0), and the
+// norms are taken too.  VEC: 16-byte loads (n a multiple of 4, staged).
+template <bool FIRST, bool VEC>
+__global__ void __launch_bounds__(kThreads, FIRST && VEC ? 2 : 3) rikfad_diag_rows_kernel(DiagParams d)
 {
-    __shared__ double s1[kWarps], s2[kWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t row = (int64_t)blockIdx.x * kWarps + warp;
-    const float inv = st->inv;
-    float f1 = 0.f, f2 = 0.f;
-    if (row < m) {
-        const float rhat = R[row] * inv;
-        // kDiagBatch loads in flight per lane, then the sums in element order
-        for (int64_t j0 = lane; j0 < n; j0 += 32 * kDiagBatch) {
-            float xv[kDiagBatch], cv[kDiagBatch];
-#pragma unroll
-            for (int k = 0; k < kDiagBatch; ++k) {
-                const int64_t j = j0 + 32 * k;
-                xv[k] = j < n ? xi[row * n + j] : 0.f;
-                cv[k] = j < n ? C[j] : 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < kDiagBatch; ++k) {
-                const float d = xv[k] - rhat * cv[k];
-                f1 = fmaf(xv[k], xv[k], f1);
-                f2 = fmaf(d, d, f2);
-            }
-        }
-    }
-    const double a1 = (double)warp_sum(f1);
-    const double a2 = (double)warp_sum(f2);
-    if (lane == 0) {
-        s1[warp] = a1;
-        s2[warp] = a2;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t1 = 0.0, t2 = 0.0;
-        for (int k = 0; k < kWarps; ++k) {
-            t1 += s1[k];
-            t2 += s2[k];
-        }
-        part[2 * blockIdx.x] = t1;
-        part[2 * blockIdx.x + 1] = t2;
-    }
-}
-
-// u = xi v, one warp per row, and per block of 8 rows the sum of u_i^2 in
-// float64 (upart[block]).  Returns at once once the iteration is done.
-__global__ void __launch_bounds__(kThreads) rikfad_diag_matvec_kernel(const float *xi, int64_t m, int64_t n,
-                                                                      const float *v, float *u, double *upart,
-                                                                      const DiagState *st)
-{
-    __shared__ double su[kWarps];
-    if (st->done)
+    extern __shared__ __align__(16) float dsm[];
+    __shared__ float2 ue[kWarps], nf[kWarps];
+    __shared__ float us[kWarps];
+    __shared__ double dd[3][kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t n = d.td.cols, m = d.td.rows;
+    wait_for_predecessor();
+    allow_successor_launch();
+    if (!FIRST && d.st->done)
         return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t row = (int64_t)blockIdx.x * kWarps + warp;
-    float acc = 0.f;
-    if (row < m) {
-        for (int64_t j0 = lane; j0 < n; j0 += 32 * kDiagBatch) {
-            float a[kDiagBatch], b[kDiagBatch];
+    const bool staged = n <= kDiagStageCols;
+    float *wacc = staged ? dsm + (n + 3) / 4 * 4 : d.wpart + (int64_t)blockIdx.x * n;
+    const float *v = staged ? dsm : FIRST ? d.C : d.v;
+    float inv = 0.f, vscale = 1.f, vbias = 0.f;
+    if (FIRST) {
+        inv = inv_denominator(row_total(d.spart, d.td), d.eps);
+        float mx = 0.f;
+        for (int64_t j = tid; j < n; j += kThreads)
+            mx = fmaxf(mx, d.C[j]);
 #pragma unroll
-            for (int k = 0; k < kDiagBatch; ++k) {
-                const int64_t j = j0 + 32 * k;
-                a[k] = j < n ? xi[row * n + j] : 0.f;
-                b[k] = j < n ? v[j] : 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < kDiagBatch; ++k)
-                acc = fmaf(a[k], b[k], acc);
-        }
-        acc = warp_sum(acc);
+        for (int o = 16; o > 0; o >>= 1)
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (lane == 0)
-            u[row] = acc;
+            us[warp] = mx;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kWarps; ++k)
+            mx = fmaxf(mx, us[k]);
+        __syncthreads();
+        const float unit = rsqrtf((float)n);
+        vscale = mx > 0.f ? unit / mx : 0.f;
+        if (!isfinite(vscale) || vscale == 0.f) {   // C = 0, not finite, or too small to scale
+            vscale = 0.f;
+            vbias = unit;
+        }
     }
-    if (lane == 0)
-        su[warp] = row < m ? (double)acc * (double)acc : 0.0;
+    // v_j: as staged, or (FIRST, not staged) from C.
+    auto first_v = [&](float c) { return vscale != 0.f ? __fmul_rn(c, vscale) : vbias; };
+    if (staged) {
+        for (int64_t j = tid; j < n; j += kThreads)
+            dsm[j] = FIRST ? first_v(d.C[j]) : d.v[j];
+    }
+    if (VEC)
+        for (int64_t j = tid; j < n / 4; j += kThreads)
+            reinterpret_cast<float4 *>(wacc)[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    else
+        for (int64_t j = tid; j < n; j += kThreads)
+            wacc[j] = 0.f;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    auto v_at = [&](int64_t j) { return FIRST && !staged ? first_v(v[j]) : v[j]; };
+    if (FIRST && blockIdx.x == 0) {     // ||v||^2 of the first iterate
+        double a = 0.0;
+        for (int64_t j = tid; j < n; j += kThreads) {
+            const double t = (double)v_at(j);
+            a += t * t;
+        }
+        a = warp_sum_f64(a);
+        if (lane == 0)
+            dd[0][warp] = a;
+        __syncthreads();
+        for (int b = tid; b < d.ncb; b += kThreads) {
+            double t = 0.0;
+            if (b == 0)
+                for (int k = 0; k < kWarps; ++k)
+                    t += dd[0][k];
+            d.v2part[b] = t;
+        }
+        __syncthreads();
+    }
+
+    const int wpr = d.wpr, rpb = kWarps / wpr;
+    const int64_t r0 = m * blockIdx.x / d.nblk, r1 = m * (blockIdx.x + 1) / d.nblk;
+    const int part = warp % wpr, sub = warp / wpr;
+    double u2 = 0.0, n1 = 0.0, n2 = 0.0;        // thread k < rpb: its rows
+    for (int64_t r = r0; r < r1; r += rpb) {
+        const int64_t row = r + sub;
+        float s = 0.f, e = 0.f, f1 = 0.f, f2 = 0.f;
+        if (row < r1) {
+            const float *x = d.xi + row * n;
+            const float rhat = FIRST ? d.R[row] * inv : 0.f;
+            if (VEC) {
+                constexpr int kU = 4;
+                const float4 *x4 = reinterpret_cast<const float4 *>(x);
+                const float4 *v4 = reinterpret_cast<const float4 *>(v);
+                const int n4 = (int)(n / 4), step = 32 * wpr;
+                float4 sv = make_float4(0.f, 0.f, 0.f, 0.f), ev = sv, g1 = sv, g2 = sv;
+                for (int q0 = part * 32 + lane; q0 < n4; q0 += step * kU) {
+                    float4 xv[kU];
+#pragma unroll
+                    for (int k = 0; k < kU; ++k)
+                        if (q0 + k * step < n4)
+                            xv[k] = x4[q0 + k * step];
+#pragma unroll
+                    for (int k = 0; k < kU; ++k) {
+                        const int q = q0 + k * step;
+                        if (q < n4) {
+                            const float4 b = v4[q];
+                            dot2(sv.x, ev.x, xv[k].x, b.x);
+                            dot2(sv.y, ev.y, xv[k].y, b.y);
+                            dot2(sv.z, ev.z, xv[k].z, b.z);
+                            dot2(sv.w, ev.w, xv[k].w, b.w);
+                            if (FIRST) {
+                                const float d0 = xv[k].x - rhat * d.C[4 * q];
+                                const float d1 = xv[k].y - rhat * d.C[4 * q + 1];
+                                const float d2 = xv[k].z - rhat * d.C[4 * q + 2];
+                                const float d3 = xv[k].w - rhat * d.C[4 * q + 3];
+                                g1.x = fmaf(xv[k].x, xv[k].x, g1.x);
+                                g1.y = fmaf(xv[k].y, xv[k].y, g1.y);
+                                g1.z = fmaf(xv[k].z, xv[k].z, g1.z);
+                                g1.w = fmaf(xv[k].w, xv[k].w, g1.w);
+                                g2.x = fmaf(d0, d0, g2.x);
+                                g2.y = fmaf(d1, d1, g2.y);
+                                g2.z = fmaf(d2, d2, g2.z);
+                                g2.w = fmaf(d3, d3, g2.w);
+                            }
+                        }
+                    }
+                }
+                s = sv.x;
+                e = ev.x;
+                add2(s, e, sv.y, ev.y);
+                add2(s, e, sv.z, ev.z);
+                add2(s, e, sv.w, ev.w);
+                f1 = (g1.x + g1.y) + (g1.z + g1.w);
+                f2 = (g2.x + g2.y) + (g2.z + g2.w);
+            } else {
+                constexpr int kU = 8;
+                const int64_t step = 32 * wpr;
+                for (int64_t j0 = part * 32 + lane; j0 < n; j0 += step * kU) {
+                    float xv[kU], vv[kU];
+#pragma unroll
+                    for (int k = 0; k < kU; ++k)
+                        if (j0 + k * step < n) {
+                            xv[k] = x[j0 + k * step];
+                            vv[k] = v_at(j0 + k * step);
+                        }
+#pragma unroll
+                    for (int k = 0; k < kU; ++k)
+                        if (j0 + k * step < n) {
+                            dot2(s, e, xv[k], vv[k]);
+                            if (FIRST) {
+                                const float t = xv[k] - rhat * d.C[j0 + k * step];
+                                f1 = fmaf(xv[k], xv[k], f1);
+                                f2 = fmaf(t, t, f2);
+                            }
+                        }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
+            const float e2 = __shfl_xor_sync(0xffffffffu, e, o);
+            add2(s, e, s2, e2);
+        }
+        if (FIRST) {
+            f1 = warp_sum(f1);
+            f2 = warp_sum(f2);
+        }
+        if (lane == 0) {
+            ue[warp] = make_float2(s, e);
+            if (FIRST)
+                nf[warp] = make_float2(f1, f2);
+        }
+        __syncthreads();
+        if (tid < rpb) {
+            float us_ = ue[tid * wpr].x, ue_ = ue[tid * wpr].y;
+            for (int k = 1; k < wpr; ++k)
+                add2(us_, ue_, ue[tid * wpr + k].x, ue[tid * wpr + k].y);
+            const double u = (double)us_ + (double)ue_;
+            u2 += u * u;
+            us[tid] = us_ + ue_;        // 0 for a row past the block's range
+            if (FIRST)
+                for (int k = 0; k < wpr; ++k) {
+                    n1 += (double)nf[tid * wpr + k].x;
+                    n2 += (double)nf[tid * wpr + k].y;
+                }
+        }
+        __syncthreads();
+        const int live = (int)(r1 - r < rpb ? r1 - r : rpb);
+        const float *x = d.xi + r * n;
+        if (VEC) {
+            const int n4 = (int)(n / 4);
+            float4 *w4 = reinterpret_cast<float4 *>(wacc);
+            for (int q = tid; q < n4; q += kThreads) {
+                float4 acc = w4[q];
+                float4 xv[kWarps];
+#pragma unroll
+                for (int k = 0; k < kWarps; ++k)
+                    if (k < live)
+                        xv[k] = reinterpret_cast<const float4 *>(x)[(int64_t)k * n4 + q];
+#pragma unroll
+                for (int k = 0; k < kWarps; ++k)
+                    if (k < live) {
+                        acc.x = fmaf(xv[k].x, us[k], acc.x);
+                        acc.y = fmaf(xv[k].y, us[k], acc.y);
+                        acc.z = fmaf(xv[k].z, us[k], acc.z);
+                        acc.w = fmaf(xv[k].w, us[k], acc.w);
+                    }
+                w4[q] = acc;
+            }
+        } else {
+            for (int64_t j = tid; j < n; j += kThreads) {
+                float acc = wacc[j];
+                float xv[kWarps];
+#pragma unroll
+                for (int k = 0; k < kWarps; ++k)
+                    if (k < live)
+                        xv[k] = x[k * n + j];
+#pragma unroll
+                for (int k = 0; k < kWarps; ++k)
+                    if (k < live)
+                        acc = fmaf(xv[k], us[k], acc);
+                wacc[j] = acc;
+            }
+        }
+    }
+    // The block's share of xi^T u (each thread the columns it owns), its sums.
+    if (staged) {
+        float *out = d.wpart + (int64_t)blockIdx.x * n;
+        if (VEC)
+            for (int64_t j = tid; j < n / 4; j += kThreads)
+                reinterpret_cast<float4 *>(out)[j] = reinterpret_cast<const float4 *>(wacc)[j];
+        else
+            for (int64_t j = tid; j < n; j += kThreads)
+                out[j] = wacc[j];
+    }
+    if (tid < kWarps) {
+        dd[0][tid] = u2;
+        dd[1][tid] = n1;
+        dd[2][tid] = n2;
+    }
+    __syncthreads();
+    if (tid < (FIRST ? 3 : 1)) {
         double t = 0.0;
         for (int k = 0; k < kWarps; ++k)
-            t += su[k];
-        upart[blockIdx.x] = t;
+            t += dd[tid][k];
+        if (tid == 0)
+            d.upart[blockIdx.x] = t;
+        else
+            d.npart[2 * blockIdx.x + tid - 1] = t;
     }
 }
 
-// wpart[g][j] = sum over the rows of row group g (blockIdx.x) of xi_ij u_i,
-// for the kThreads columns of tile blockIdx.y (one thread per column, rows
-// in order).  Returns at once once the iteration is done.
-__global__ void __launch_bounds__(kThreads) rikfad_diag_matvec_t_kernel(const float *xi, int64_t m, int64_t n,
-                                                                        const float *u, float *wpart,
-                                                                        const DiagState *st)
+// Column kernel: cpb columns a block, 32 at a time.  The next iterate v =
+// (xi^T u) ||v||^2 / ||u||^2 (whose length stays near the last one's and equals
+// it once converged): warp k adds the row blocks k, k + 8, ... in order, then
+// warp 0 the eight warp sums; its squares go to the other half of v2part.
+// Block 0 forms the quotient and tests convergence: |sigma^2 - previous| <= tol
+// sigma^2 from the second iteration on, or max_iters, or nothing left to
+// iterate on.
+__global__ void __launch_bounds__(kThreads) rikfad_diag_cols_kernel(DiagParams d)
 {
-    if (st->done)
-        return;
-    const int64_t rpg = diag_rows_per_group(m);
-    const int64_t r0 = (int64_t)blockIdx.x * rpg;
-    const int64_t r1 = r0 + rpg < m ? r0 + rpg : m;
-    const int64_t j = (int64_t)blockIdx.y * kThreads + threadIdx.x;
-    if (j >= n)
-        return;
-    float acc = 0.f;
-    for (int64_t i0 = r0; i0 < r1; i0 += kDiagBatch) {
-        float a[kDiagBatch], b[kDiagBatch];
-#pragma unroll
-        for (int k = 0; k < kDiagBatch; ++k) {
-            const int64_t i = i0 + k;
-            a[k] = i < r1 ? xi[i * n + j] : 0.f;
-            b[k] = i < r1 ? u[i] : 0.f;
-        }
-#pragma unroll
-        for (int k = 0; k < kDiagBatch; ++k)
-            acc = fmaf(a[k], b[k], acc);
-    }
-    wpart[(int64_t)blockIdx.x * n + j] = acc;
-}
-
-// w_j = sum over the row groups of wpart[g][j] for the 32 columns of block
-// blockIdx.x (kDiagFinThreads threads): warp k adds groups k, k + 32,
-// k + 64, ... in order, then warp 0 adds the 32 warp sums in warp order.  w
-// goes to w, and the block's sum of w_j^2 (float64) to wsq[blockIdx.x].
-// Returns at once once the iteration is done.
-__global__ void __launch_bounds__(kDiagFinThreads) rikfad_diag_colsum_kernel(const float *wpart, int nb,
-                                                                             int64_t n, float *w, double *wsq,
-                                                                             const DiagState *st)
-{
-    constexpr int kColWarps = kDiagFinThreads / 32;
-    __shared__ float part[kColWarps][32];
-    if (st->done)
-        return;
+    constexpr int kU = 8;
+    __shared__ float part[kWarps][32];
+    __shared__ double tot[4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t j = (int64_t)blockIdx.x * 32 + lane;
-    float acc = 0.f;
-    if (j < n) {
-        for (int g0 = warp; g0 < nb; g0 += kColWarps * kDiagBatch) {
-            float t[kDiagBatch];
+    const int64_t n = d.td.cols;
+    wait_for_predecessor();
+    allow_successor_launch();
+    if (d.st->done)
+        return;
+    const int it = d.st->it + 1;
+    // Totals, each by one warp: ||u||^2, ||v||^2, and (block 0, first iteration) the norms.
+    if (warp < 2 || (it == 1 && blockIdx.x == 0 && warp < 4)) {
+        const double *src = warp == 0 ? d.upart : warp == 1 ? d.v2part + (int64_t)d.parity * d.ncb : d.npart + (warp - 2);
+        const int cnt = warp == 1 ? d.ncb : d.nblk, stride = warp < 2 ? 1 : 2;
+        double a = 0.0;
+        for (int b = lane; b < cnt; b += 32)
+            a += src[b * stride];
+        a = warp_sum_f64(a);
+        if (lane == 0)
+            tot[warp] = a;
+    }
+    double q = 0.0;             // warp 0: squares of the next iterate
+    for (int64_t c0 = 0; c0 < d.cpb; c0 += 32) {
+        const int64_t j = (int64_t)blockIdx.x * d.cpb + c0 + lane;
+        float acc = 0.f;
+        if (j < n) {
+            for (int g0 = warp; g0 < d.nblk; g0 += kWarps * kU) {
+                float t[kU];
 #pragma unroll
-            for (int k = 0; k < kDiagBatch; ++k) {
-                const int g = g0 + k * kColWarps;
-                t[k] = g < nb ? wpart[(int64_t)g * n + j] : 0.f;
+                for (int k = 0; k < kU; ++k) {
+                    const int g = g0 + k * kWarps;
+                    t[k] = g < d.nblk ? d.wpart[(int64_t)g * n + j] : 0.f;
+                }
+#pragma unroll
+                for (int k = 0; k < kU; ++k)
+                    acc += t[k];
             }
+        }
+        __syncthreads();        // warp 0 has read the last 32 columns' sums
+        part[warp][lane] = acc;
+        __syncthreads();
+        if (warp == 0 && j < n) {
+            float sum = 0.f;
 #pragma unroll
-            for (int k = 0; k < kDiagBatch; ++k)
-                acc += t[k];
+            for (int k = 0; k < kWarps; ++k)
+                sum += part[k][lane];
+            const float vn = tot[0] > 0.0 ? (float)((double)sum * (tot[1] / tot[0])) : 0.f;
+            d.v[j] = vn;
+            q += (double)vn * (double)vn;
         }
     }
-    part[warp][lane] = acc;
-    __syncthreads();
-    if (warp == 0) {
-        float sum = 0.f;
-#pragma unroll 8
-        for (int k = 0; k < kColWarps; ++k)
-            sum += part[k][lane];
-        if (j < n)
-            w[j] = sum;
-        const double q = warp_sum_f64(j < n ? (double)sum * (double)sum : 0.0);
-        if (lane == 0)
-            wsq[blockIdx.x] = q;
-    }
-}
-
-// End of one power iteration, one block: ||w||^2 from the column blocks'
-// partials, sigma^2 = ||u||^2 (the Rayleigh quotient of xi^T xi at the unit
-// v) from the row blocks' partials, the next iterate v = w / ||w||, and the
-// convergence test |sigma^2 - previous| <= tol sigma^2 (from the second
-// iteration on); done after max_iters iterations or when w = 0.
-__global__ void __launch_bounds__(kDiagFinThreads) rikfad_diag_iterate_kernel(
-    const float *w, int64_t n, const double *wsq, int nbw, const double *upart, int nbu, float *v,
-    DiagState *st, double tol, int max_iters)
-{
-    __shared__ double scratch[kDiagFinThreads / 32 + 1];
-    __shared__ double s_scale;
-    if (st->done)
+    if (warp != 0)
         return;
-    double a = 0.0;
-    for (int b = threadIdx.x; b < nbw; b += kDiagFinThreads)
-        a += wsq[b];
-    const double w2 = block_sum_f64<kDiagFinThreads>(a, scratch);
-    double c = 0.0;
-    for (int b = threadIdx.x; b < nbu; b += kDiagFinThreads)
-        c += upart[b];
-    const double u2 = block_sum_f64<kDiagFinThreads>(c, scratch);
-    if (threadIdx.x == 0)
-        s_scale = w2 > 0.0 ? 1.0 / sqrt(w2) : 0.0;
-    __syncthreads();
-    if (w2 > 0.0) {
-        // The product in float64, rounded once (scaled in float32 the quotient
-        // seldom settled to a 1e-10 convergence test).
-        const double sc = s_scale;
-        for (int64_t j = threadIdx.x; j < n; j += kDiagFinThreads)
-            v[j] = (float)((double)w[j] * sc);
-    }
-    if (threadIdx.x == 0) {
-        const double prev = st->sigma2;
-        const int it = st->it + 1;
-        st->it = it;
-        st->sigma2 = u2;
-        st->w2 = w2;
-        if (w2 == 0.0 || it >= max_iters || (it > 1 && fabs(u2 - prev) <= tol * u2))
-            st->done = 1;
+    q = warp_sum_f64(q);
+    if (lane == 0)
+        d.v2part[(int64_t)(d.parity ^ 1) * d.ncb + blockIdx.x] = q;
+    if (blockIdx.x == 0 && lane == 0) {
+        const double u2 = tot[0], v2 = tot[1];
+        DiagState s = *d.st;
+        const double prev = s.sigma2;
+        if (it == 1) {
+            s.f2 = tot[2];
+            s.e2 = tot[3];
+        }
+        s.it = it;
+        // An iterate that underflowed to zero leaves the last quotient.
+        if (v2 > 0.0 && (u2 > 0.0 || it == 1))
+            s.sigma2 = u2 / v2;
+        s.done = !(u2 > 0.0) || it >= d.max_iters || (it > 1 && fabs(s.sigma2 - prev) <= d.tol * s.sigma2);
+        *d.st = s;
+        if (s.done || d.last)
+            *d.host = s;
     }
 }
 

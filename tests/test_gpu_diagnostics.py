@@ -134,3 +134,37 @@ def test_diagnostics_refused_for_other_handles():
         opt.friction_diagnostics(0)
     assert e.value.code == rikfad.ERR_STATE
     opt.close()
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 4096), (151, 12), (152, 4097), (303, 4100), (608, 5), (1216, 33),
+                                 (3700, 64), (65, 20000)])
+def test_diagnostics_at_the_edges_of_the_kernels(m, n):
+    """One warp per row to eight (m around 1216, 608, 304), several passes per
+    block, 16-byte and single loads, staged and unstaged iterates (4096
+    columns), more than one batch of iterations, and a cut at max_iters.
+
+    sigma_1: u is compensated (n 2^-48), the iterate's rounding enters squared,
+    and the quotient is converged to tol / (1 - ratio) < 1e-10: 1e-9.  Norms:
+    float32 row sums of ceil(n / 32) terms a lane and 8 levels, each term's
+    rounding included (xi~ itself is three roundings of a product)."""
+    inp = workloads.ModelInputs([(m, n)], seed=44, g_std=1e-2)
+    run = DeviceRun([(m, n)], HP, True, inp.X, inp.P, method="ikfad_shadow")
+    zero = run.opt.friction_diagnostics(0)              # xi = 0, C = 0
+    assert zero[:5] == (0.0,) * 5 and zero[5] == 1.0
+    for k in range(3):
+        run.set_grads(inp.grads(k))
+        run.step(0.1)
+    err, floor, sr, s1, frob, iters = run.opt.friction_diagnostics(0, max_iters=500, tol=1e-12)
+    XI = run.opt.get_friction(0).astype(np.float64)
+    R, C = (a.astype(np.float64) for a in run.opt.get_factors(0))
+    e_ref, f_ref, sr_ref, s1_ref, frob_ref = friction_metrics(XI, R, C, HP.eps_stab)
+    u = 2.0 ** -24 * (-(-n // 32) + 10)
+    assert iters < 500
+    assert abs(s1 - s1_ref) <= 1e-9 * s1_ref, (s1, s1_ref, iters)
+    assert abs(frob - frob_ref) <= u * frob_ref, (frob, frob_ref)
+    assert abs(sr - sr_ref) <= 3 * u * sr_ref, (sr, sr_ref)
+    # ||xi - xi~||: its own sum's rounding, and xi~'s (8 roundings with 1^T R's tree) relative to ||xi~||
+    assert abs(err - e_ref) <= u * (2 * e_ref + 1) , (err, e_ref)
+    cut = run.opt.friction_diagnostics(0, max_iters=1)
+    assert cut[5] == 1.0 and cut[3] <= s1 * (1 + 1e-9)
+    run.close()
