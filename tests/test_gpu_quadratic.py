@@ -254,3 +254,40 @@ def test_prefactor_table_matches_oracle_and_paper():
             assert abs(q[0] / ref - 1) < 1e-3, (name, al, mu, ep, q[0], ref)
         spread = np.median(v.max(axis=0) / v.min(axis=0))
         assert spread < (1.3 if name == "tE_over_alpha_mu" else 1.2), (name, spread)
+
+
+LANE_SHAPES = [(1, 1), (1, 2), (2, 2), (4, 1), (2, 3), (3, 3), (4, 4), (7, 1), (2, 8), (3, 6), (7, 3), (4, 8), (8, 4),
+               (5, 6), (6, 5), (5, 5), (1, 9), (13, 2), (2, 16), (9, 3), (3, 10), (17, 1), (1, 32)]
+
+
+@pytest.mark.parametrize("m,n", LANE_SHAPES)
+def test_large_batches_match_oracle(m, n):
+    """Batches that take one lane per row (or column), for every number of
+    lanes and of elements per lane: ragged last warps, records at the first,
+    middle and last steps, gamma > 0, factors that start nonzero, large enough
+    for exp(z) - 1 beyond the series (the first instance) and all zero (the
+    second, with eps = 0 until its first step).  61 steps, at the bounds of this
+    file; the same instance gives the same bits wherever it lies in the batch."""
+    seeds, batch = list(range(50, 61)), 12163
+    A, X, P = workloads.dense_quadratic_batch(m, n, seeds)
+    rng = np.random.default_rng(8)
+    R = rng.uniform(0.1, 1.0, (len(seeds), m)).astype(np.float32)
+    C = rng.uniform(0.1, 1.0, (len(seeds), n)).astype(np.float32)
+    R[0] *= 300.0
+    C[0] *= 300.0
+    R[1], C[1] = 0.0, 0.0
+    idx = np.arange(batch) % len(seeds)
+    hp = HParams(1.0, 1.0, 0.05, 0.0)
+    rec = [0, 1, 30, 61]
+    st = _gpu_state(A[idx], X[idx], P[idx], R[idx], C[idx])
+    Eg = _run(st, 61, rec, hp)
+    got = {k: st[k].cpu().numpy() for k in "XPRC"}
+    for s in range(len(seeds)):
+        E, Xo, Po, Ro, Co = _oracle(A[s], X[s], P[s], 61, rec, hp, R[s], C[s])
+        assert np.all(np.abs(Eg[:, s] - E) <= E_RTOL * E), (s, Eg[:, s], E)
+        for k, r in zip("XPRC", (Xo, Po, Ro, Co)):
+            compare(k, got[k][s], r, S_RTOL, 1.0)
+        same = np.nonzero(idx == s)[0]
+        assert np.all(Eg[:, same] == Eg[:, [s]])
+        for k in "XPRC":
+            assert np.all(got[k][same] == got[k][s]), (k, s)
