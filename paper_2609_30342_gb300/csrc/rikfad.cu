@@ -158,6 +158,7 @@ struct rikfad_handle_s {
     int32_t *d_block_piece = nullptr;
     int64_t *d_slot_off = nullptr;
     FinItemDev *d_fin = nullptr;
+    TileDev *d_tiles = nullptr;
     float *d_fac = nullptr;
     float *d_rowpart = nullptr;
     float *d_colpart = nullptr;
@@ -339,7 +340,7 @@ bool hparams_ok(const rikfad_hparams &hp, std::string &why)
 void release(rikfad_handle h)
 {
     for (void *p : {(void *)h->d_tensors, (void *)h->d_panels, (void *)h->d_pieces, (void *)h->d_block_piece,
-                    (void *)h->d_slot_off, (void *)h->d_fin, (void *)h->d_fac, (void *)h->d_rowpart,
+                    (void *)h->d_slot_off, (void *)h->d_fin, (void *)h->d_tiles, (void *)h->d_fac, (void *)h->d_rowpart,
                     (void *)h->d_colpart, (void *)h->d_spart, (void *)h->d_den, (void *)h->d_guard,
                     (void *)h->d_checks, (void *)h->d_diag_v, (void *)h->d_diag_wpart,
                     (void *)h->d_diag_norms, (void *)h->d_diag_upart, (void *)h->d_diag_v2part,
@@ -425,6 +426,7 @@ CheckBounds bounds(const rikfad_handle h)
     cb.nblocks = p.nblocks;
     cb.nfin = (int32_t)p.fin_items.size();
     cb.nslots = (int32_t)p.slot_off.size();
+    cb.ntiles = (int32_t)p.tiles.size();
     cb.fac_floats = p.fac_floats;
     cb.rowpart_floats = p.rowpart_floats;
     cb.colpart_floats = p.colpart_floats;
@@ -516,8 +518,7 @@ int canonical(rikfad_handle h, const float *const *src, float *const *dst, bool 
         CanonParams c{};
         c.tensors = h->d_tensors;
         c.panels = h->d_panels;
-        c.pieces = h->d_pieces;
-        c.block_piece = h->d_block_piece;
+        c.tiles = h->d_tiles;
         c.src = (const float *const *)h->canon_ptrs.dev;
         c.dst = (float *const *)(h->canon_ptrs.dev + T);
         c.fac = h->d_fac;
@@ -526,7 +527,7 @@ int canonical(rikfad_handle h, const float *const *src, float *const *dst, bool 
         c.damp_prev = (float)std::exp(-h->hp.gamma * h->pending_step);
         c.eps = (float)h->hp.eps_stab;
         c.chk = bounds(h);
-        RK_CUDA(launch_pdl(rikfad_canonical_kernel, h->plan.nblocks, kThreads, stream, c),
+        RK_CUDA(launch_pdl(rikfad_canonical_kernel, (int)h->plan.tiles.size(), kThreads, stream, c),
                 "launch rikfad_canonical_kernel");
     }
     if (commit)
@@ -708,6 +709,7 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     if (!rc) rc = upload(&h->d_block_piece, p.block_piece, ws);
     if (!rc) rc = upload(&h->d_slot_off, p.slot_off, ws);
     if (!rc) rc = upload(&h->d_fin, p.fin_items, ws);
+    if (!rc) rc = upload(&h->d_tiles, p.tiles, ws);
     size_t state = 0;
     if (!rc) rc = alloc_zero(&h->d_fac, p.fac_floats, state);
     if (!rc) rc = alloc_zero(&h->d_rowpart, p.rowpart_floats, ws);
@@ -870,6 +872,7 @@ RIKFAD_API int rikfad_step(rikfad_handle h, double step, float *const *x, const 
         a.panels = h->d_panels;
         a.pieces = h->d_pieces;
         a.block_piece = h->d_block_piece;
+        a.tiles = h->d_tiles;
         a.xptr = (float *const *)h->step_ptrs.dev;
         a.gptr = (const void *const *)(h->step_ptrs.dev + T);
         a.pptr = (float *const *)(h->step_ptrs.dev + 2 * T);
@@ -906,9 +909,15 @@ RIKFAD_API int rikfad_step(rikfad_handle h, double step, float *const *x, const 
                 launch_sweep<float>(a, sp, reuse, h->sweep_blocks, s);
             RK_CUDA(cudaGetLastError(), "launch rikfad_sweep_kernel");
         } else {
-            RK_CUDA(launch_pdl(step_kernel(h->grad_bytes, reuse, h->shadow, h->ragged), h->plan.nblocks,
-                               kThreads, s, a),
-                    "launch rikfad_step_kernel");
+            if (h->plan.elements_only)
+                RK_CUDA(launch_pdl(h->grad_bytes == 2 ? rikfad_elements_kernel<__nv_bfloat16>
+                                                      : rikfad_elements_kernel<float>,
+                                   (int)h->plan.tiles.size(), kThreads, s, a),
+                        "launch rikfad_elements_kernel");
+            else
+                RK_CUDA(launch_pdl(step_kernel(h->grad_bytes, reuse, h->shadow, h->ragged), h->plan.nblocks,
+                                   kThreads, s, a),
+                        "launch rikfad_step_kernel");
         }
     }
     if (ev)

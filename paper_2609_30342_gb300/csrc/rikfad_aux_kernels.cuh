@@ -17,8 +17,7 @@ struct DenParams {
 struct CanonParams {
     const TensorDev *tensors;
     const PanelDev *panels;
-    const PieceDev *pieces;
-    const int32_t *block_piece;
+    const TileDev *tiles;
     const float *const *src;
     float *const *dst;
     const float *fac;
@@ -196,98 +195,159 @@ __global__ void __launch_bounds__(kFinThreads) rikfad_finalize_kernel(FinParams 
 // dst = src exp(-(h_prev/2) xi~) e^{-gamma h_prev} for matrices (the same
 // expression, in the same rounding order, as the start of the next step);
 // vectors already hold P_{n+1} and are copied when dst != src.
-__global__ void __launch_bounds__(kThreads) rikfad_canonical_kernel(CanonParams c)
+//
+// Bound by HBM (8 B an element).  No sums cross rows, so a block takes one tile
+// of a panel's rows, in memory order; its first loads are issued before C is
+// staged.  GPT2-S (1.0 GB): 147 us (6.8 TB/s), against 155 from two persistent
+// blocks per SM with a contiguous share each, one row per warp.  A narrow
+// matrix's tile is taken as a run of elements: 400000 x 64 in 37 us instead of
+// 156, 1000000 x 8 in 16 instead of 287; 64-column panels beside wide ones gain
+// from the order (eight layers of width 1600: 1394 -> 388 us).
+__device__ __forceinline__ void canonical_copy(const float *S, float *D, int64_t n)
+{
+    for (int64_t e = threadIdx.x; e < n; e += kThreads)
+        D[e] = S[e];
+}
+
+__global__ void __launch_bounds__(kThreads, 4) rikfad_canonical_kernel(CanonParams c)
 {
     __shared__ float Cs[kPanelMax];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (!RK_DEV_CHECK(c.chk, (int)blockIdx.x < c.chk.ntiles, kChkBlock))
+        return;
+    const TileDev tile = c.tiles[blockIdx.x];
+    PieceDev pc{};
+    pc.kind = tile.panel < 0 ? kElements : kMatrixRows;
+    pc.tensor = tile.tensor;
+    pc.panel = tile.panel;
+    if (!piece_tensor_ok(c.chk, pc))
+        return;
+    const TensorDev td = c.tensors[pc.tensor];
+    pc.begin = tile.begin;
     wait_for_predecessor();
     allow_successor_launch();
-    if (!RK_DEV_CHECK(c.chk, (int)blockIdx.x < c.chk.nblocks, kChkBlock))
+    const float *S = c.src[pc.tensor];
+    float *D = c.dst[pc.tensor];
+    if (pc.kind == kElements) {
+        pc.end = tile.begin + kTileElems < td.rows ? tile.begin + kTileElems : td.rows;
+        if (S != D && vector_piece_ok(c.chk, pc, td, D, nullptr, S, false))
+            canonical_copy(S + pc.begin, D + pc.begin, pc.end - pc.begin);
         return;
-    const int q0 = c.block_piece[blockIdx.x], q1 = c.block_piece[blockIdx.x + 1];
-    if (!block_ok(c.chk, blockIdx.x, q0, q1))
+    }
+    if (!piece_panel_ok(c.chk, pc, td))
         return;
-    for (int q = q0; q < q1; ++q) {
-        const PieceDev pc = c.pieces[q];
-        if (!piece_tensor_ok(c.chk, pc))
-            continue;
-        const TensorDev td = c.tensors[pc.tensor];
-        const float *S = c.src[pc.tensor];
-        float *D = c.dst[pc.tensor];
-        if (pc.kind == kElements) {
-            if (S != D && vector_piece_ok(c.chk, pc, td, D, nullptr, S, false))
-                for (int64_t e = pc.begin + threadIdx.x; e < pc.end; e += kThreads)
-                    D[e] = S[e];
-            continue;
-        }
-        if (!piece_panel_ok(c.chk, pc, td))
-            continue;
-        const PanelDev pd = c.panels[pc.panel];
-        if (!matrix_piece_ok(c.chk, pc, td, pd, D, nullptr, S, false))
-            continue;
-        if (td.full) {      // element-wise friction: P already holds P_{n+1}
-            if (S != D)
-                for (int64_t row = pc.begin + warp; row < pc.end; row += kWarps)
-                    for (int j = lane; j < pd.width; j += 32)
-                        D[row * td.cols + pd.col0 + j] = S[row * td.cols + pd.col0 + j];
-            continue;
-        }
-        const float *C = c.fac + td.fac_off + td.rows + pd.col0;
-        for (int j = threadIdx.x; j < pd.width; j += kThreads)
-            Cs[j] = C[j];
-        const float inv = inv_denominator(row_total(c.spart, td), c.eps);
-        __syncthreads();
-        const float *R = c.fac + td.fac_off;
-        for (int64_t row = pc.begin + warp; row < pc.end; row += kWarps) {
-            const float a_prev = c.ex_prev * (R[row] * inv);
-            const int64_t base = row * td.cols + pd.col0;
-            if (td.vec) {
-                // 16-byte aligned rows and panels: the whole panel row is
-                // loaded first (at most kPanelMax / 128 float4 per lane), so
-                // every load is in flight before the first in-place store.
-                constexpr int kV = kPanelMax / 128;
-                const float4 *s4 = reinterpret_cast<const float4 *>(S + base);
-                float4 *d4 = reinterpret_cast<float4 *>(D + base);
-                const int w4 = pd.width / 4;
-                float4 v[kV];
+    const PanelDev pd = c.panels[pc.panel];
+    pc.end = tile.begin + pd.tile_rows < td.rows ? tile.begin + pd.tile_rows : td.rows;
+    if (!matrix_piece_ok(c.chk, pc, td, pd, D, nullptr, S, false))
+        return;
+    if (td.full) {      // element-wise friction: P already holds P_{n+1}
+        if (S != D)
+            for (int64_t row = pc.begin + warp; row < pc.end; row += kWarps)
+                for (int j = lane; j < pd.width; j += 32)
+                    D[row * td.cols + pd.col0 + j] = S[row * td.cols + pd.col0 + j];
+        return;
+    }
+    const float *C = c.fac + td.fac_off + td.rows + pd.col0;
+    const float *R = c.fac + td.fac_off;
+    // 16-byte aligned rows and panels: a whole panel row (at most kPanelMax /
+    // 128 float4 per lane) is loaded before the first in-place store.
+    constexpr int kV = kPanelMax / 128;
+    const int w4 = pd.width / 4;
+    float4 v[kV];
+    auto load_row = [&](int64_t row) {
+        const float4 *s4 = reinterpret_cast<const float4 *>(S + row * td.cols + pd.col0);
 #pragma unroll
-                for (int k = 0; k < kV; ++k)
-                    if (lane + 32 * k < w4)
-                        v[k] = __ldcs(s4 + lane + 32 * k);
+        for (int k = 0; k < kV; ++k)
+            if (lane + 32 * k < w4)
+                v[k] = __ldcs(s4 + lane + 32 * k);
+    };
+    // A narrow matrix (one panel): its tile is a run of elements, of which every
+    // lane takes its share whatever the rows' width.
+    const bool flat = td.vec && td.npanels == 1 && pd.width <= 128;
+    const int n4 = (int)(pc.end - pc.begin) * w4;       // flat: float4 of the tile
+    const float4 *t4 = reinterpret_cast<const float4 *>(S + pc.begin * td.cols);
+    auto load_flat = [&](int q0) {
 #pragma unroll
-                for (int k = 0; k < kV; ++k) {
-                    const int j4 = lane + 32 * k;
-                    if (j4 < w4) {
-                        const int j = 4 * j4;
-                        v[k].x = (v[k].x * exp2f(a_prev * Cs[j])) * c.damp_prev;
-                        v[k].y = (v[k].y * exp2f(a_prev * Cs[j + 1])) * c.damp_prev;
-                        v[k].z = (v[k].z * exp2f(a_prev * Cs[j + 2])) * c.damp_prev;
-                        v[k].w = (v[k].w * exp2f(a_prev * Cs[j + 3])) * c.damp_prev;
-                        __stcs(d4 + j4, v[k]);
-                    }
-                }
-            } else {
-                // Rows at any element address: 256 columns' loads before the
-                // first in-place store (one load in flight per lane ran at a
-                // fraction of the bandwidth, as in matrix_piece_ragged).
-                constexpr int kU = 8;
-#pragma unroll 1
-                for (int j0 = lane; j0 < pd.width; j0 += 32 * kU) {
-                    float v[kU];
+        for (int k = 0; k < kV; ++k)
+            if (q0 + 32 * k < n4)
+                v[k] = __ldcs(t4 + q0 + 32 * k);
+    };
+    int64_t row = pc.begin + warp;
+    float r = 0.f;
+    if (flat) {
+        load_flat(warp * 32 * kV + lane);
+    } else if (row < pc.end) {
+        if (td.vec)
+            load_row(row);
+        r = R[row];
+    }
+    for (int j = threadIdx.x; j < pd.width; j += kThreads)
+        Cs[j] = C[j];
+    const float inv = inv_denominator(row_total(c.spart, td), c.eps);
+    __syncthreads();
+    if (flat) {
+        float4 *d4 = reinterpret_cast<float4 *>(D + pc.begin * td.cols);
+        for (int q0 = warp * 32 * kV + lane; q0 < n4; q0 += kThreads * kV) {
+            if (q0 >= kThreads * kV)
+                load_flat(q0);
 #pragma unroll
-                    for (int u = 0; u < kU; ++u)
-                        if (j0 + 32 * u < pd.width)
-                            v[u] = __ldcs(S + base + j0 + 32 * u);
-#pragma unroll
-                    for (int u = 0; u < kU; ++u) {
-                        const int j = j0 + 32 * u;
-                        if (j < pd.width)
-                            __stcs(D + base + j, (v[u] * exp2f(a_prev * Cs[j])) * c.damp_prev);
-                    }
+            for (int k = 0; k < kV; ++k) {
+                const unsigned q = q0 + 32 * k;
+                if (q < (unsigned)n4) {
+                    const unsigned i = q / (unsigned)w4, j = 4 * (q - i * w4);
+                    const float a_prev = c.ex_prev * (R[pc.begin + i] * inv);
+                    v[k].x = (v[k].x * exp2f(a_prev * Cs[j])) * c.damp_prev;
+                    v[k].y = (v[k].y * exp2f(a_prev * Cs[j + 1])) * c.damp_prev;
+                    v[k].z = (v[k].z * exp2f(a_prev * Cs[j + 2])) * c.damp_prev;
+                    v[k].w = (v[k].w * exp2f(a_prev * Cs[j + 3])) * c.damp_prev;
+                    __stcs(d4 + q, v[k]);
                 }
             }
         }
-        __syncthreads();
+        return;
+    }
+    for (; row < pc.end; row += kWarps) {
+        const int64_t base = row * td.cols + pd.col0;
+        if (row >= pc.begin + kWarps) {
+            if (td.vec)
+                load_row(row);
+            r = R[row];
+        }
+        const float a_prev = c.ex_prev * (r * inv);
+        if (td.vec) {
+            float4 *d4 = reinterpret_cast<float4 *>(D + base);
+#pragma unroll
+            for (int k = 0; k < kV; ++k) {
+                const int j4 = lane + 32 * k;
+                if (j4 < w4) {
+                    const int j = 4 * j4;
+                    v[k].x = (v[k].x * exp2f(a_prev * Cs[j])) * c.damp_prev;
+                    v[k].y = (v[k].y * exp2f(a_prev * Cs[j + 1])) * c.damp_prev;
+                    v[k].z = (v[k].z * exp2f(a_prev * Cs[j + 2])) * c.damp_prev;
+                    v[k].w = (v[k].w * exp2f(a_prev * Cs[j + 3])) * c.damp_prev;
+                    __stcs(d4 + j4, v[k]);
+                }
+            }
+        } else {
+            // Rows at any element address: 256 columns' loads before the first
+            // in-place store (one load in flight per lane ran at a fraction of
+            // the bandwidth, as in matrix_piece_ragged).
+            constexpr int kU = 8;
+#pragma unroll 1
+            for (int j0 = lane; j0 < pd.width; j0 += 32 * kU) {
+                float u8[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (j0 + 32 * u < pd.width)
+                        u8[u] = __ldcs(S + base + j0 + 32 * u);
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int j = j0 + 32 * u;
+                    if (j < pd.width)
+                        __stcs(D + base + j, (u8[u] * exp2f(a_prev * Cs[j])) * c.damp_prev);
+                }
+            }
+        }
     }
 }
 

@@ -24,6 +24,7 @@ constexpr int kChunk = 256;          // columns one warp covers per pass (32 lan
 constexpr int kFinThreads = 256;     // threads of the finalise kernel (= rows per partial sum)
 constexpr int kFinColChunk = 32;     // columns per split column item (8 warps share its slots)
 constexpr int kFinSplitSlots = 8;    // panels with more slots than this get split column items
+constexpr int kTileElems = 2048;     // elements of a tile (8 per thread of a block)
 constexpr int kElemGranule = 8;      // element pieces start on multiples of 8 elements
 constexpr int64_t kMinBlockBytes = 64 * 1024;   // smallest share worth a block
 // The planner balances blocks on time, not bytes alone: each row of a matrix
@@ -66,6 +67,17 @@ struct PanelDev {
     int32_t nch;          // ceil(width / kChunk)
     int32_t slot_begin;   // column partial slots of this panel: [slot_begin, slot_end)
     int32_t slot_end;
+    int32_t tile_rows;    // rows of this panel's tiles
+};
+
+// One small block's work in a pass that carries no sums from row to row: up
+// to tile_rows rows of a panel, or kTileElems elements of a vector.  Tiles are
+// in memory order (rows before panels), and the hardware hands out blocks in
+// index order, so the whole GPU streams through a narrow window of HBM.
+struct TileDev {
+    int32_t tensor;
+    int32_t panel;        // -1: vector
+    int64_t begin;        // first row or element
 };
 
 struct PieceDev {
@@ -99,6 +111,7 @@ struct CheckBounds {
     int32_t nblocks;
     int32_t nfin;
     int32_t nslots;
+    int32_t ntiles;
     int64_t fac_floats;
     int64_t rowpart_floats;
     int64_t colpart_floats;
