@@ -116,7 +116,8 @@ struct ImageHeader {
     int64_t fac_floats;
     double alpha, mu, gamma, eps_stab;
 };
-static_assert(sizeof(ImageHeader) <= kImageHeader, "header too large");
+static_assert(sizeof(ImageHeader) == sizeof(HeaderParams::words) && sizeof(ImageHeader) <= kImageHeader,
+              "header size");
 
 // A device table of per-tensor pointers, uploaded only when it changes.
 struct PtrTable {
@@ -158,7 +159,7 @@ struct rikfad_handle_s {
     int32_t *d_block_piece = nullptr;
     int64_t *d_slot_off = nullptr;
     FinItemDev *d_fin = nullptr;
-    TileDev *d_tiles = nullptr;
+    TileGroupDev *d_tile_groups = nullptr;
     float *d_fac = nullptr;
     float *d_rowpart = nullptr;
     float *d_colpart = nullptr;
@@ -340,7 +341,7 @@ bool hparams_ok(const rikfad_hparams &hp, std::string &why)
 void release(rikfad_handle h)
 {
     for (void *p : {(void *)h->d_tensors, (void *)h->d_panels, (void *)h->d_pieces, (void *)h->d_block_piece,
-                    (void *)h->d_slot_off, (void *)h->d_fin, (void *)h->d_tiles, (void *)h->d_fac, (void *)h->d_rowpart,
+                    (void *)h->d_slot_off, (void *)h->d_fin, (void *)h->d_tile_groups, (void *)h->d_fac, (void *)h->d_rowpart,
                     (void *)h->d_colpart, (void *)h->d_spart, (void *)h->d_den, (void *)h->d_guard,
                     (void *)h->d_checks, (void *)h->d_diag_v, (void *)h->d_diag_wpart,
                     (void *)h->d_diag_norms, (void *)h->d_diag_upart, (void *)h->d_diag_v2part,
@@ -426,7 +427,7 @@ CheckBounds bounds(const rikfad_handle h)
     cb.nblocks = p.nblocks;
     cb.nfin = (int32_t)p.fin_items.size();
     cb.nslots = (int32_t)p.slot_off.size();
-    cb.ntiles = (int32_t)p.tiles.size();
+    cb.ngroups = (int32_t)p.tile_groups.size();
     cb.fac_floats = p.fac_floats;
     cb.rowpart_floats = p.rowpart_floats;
     cb.colpart_floats = p.colpart_floats;
@@ -518,7 +519,7 @@ int canonical(rikfad_handle h, const float *const *src, float *const *dst, bool 
         CanonParams c{};
         c.tensors = h->d_tensors;
         c.panels = h->d_panels;
-        c.tiles = h->d_tiles;
+        c.groups = h->d_tile_groups;
         c.src = (const float *const *)h->canon_ptrs.dev;
         c.dst = (float *const *)(h->canon_ptrs.dev + T);
         c.fac = h->d_fac;
@@ -527,7 +528,7 @@ int canonical(rikfad_handle h, const float *const *src, float *const *dst, bool 
         c.damp_prev = (float)std::exp(-h->hp.gamma * h->pending_step);
         c.eps = (float)h->hp.eps_stab;
         c.chk = bounds(h);
-        RK_CUDA(launch_pdl(rikfad_canonical_kernel, (int)h->plan.tiles.size(), kThreads, stream, c),
+        RK_CUDA(launch_pdl(rikfad_canonical_kernel, (int)h->plan.tile_groups.size() * kTileGroup, kThreads, stream, c),
                 "launch rikfad_canonical_kernel");
     }
     if (commit)
@@ -709,7 +710,7 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     if (!rc) rc = upload(&h->d_block_piece, p.block_piece, ws);
     if (!rc) rc = upload(&h->d_slot_off, p.slot_off, ws);
     if (!rc) rc = upload(&h->d_fin, p.fin_items, ws);
-    if (!rc) rc = upload(&h->d_tiles, p.tiles, ws);
+    if (!rc) rc = upload(&h->d_tile_groups, p.tile_groups, ws);
     size_t state = 0;
     if (!rc) rc = alloc_zero(&h->d_fac, p.fac_floats, state);
     if (!rc) rc = alloc_zero(&h->d_rowpart, p.rowpart_floats, ws);
@@ -872,7 +873,7 @@ RIKFAD_API int rikfad_step(rikfad_handle h, double step, float *const *x, const 
         a.panels = h->d_panels;
         a.pieces = h->d_pieces;
         a.block_piece = h->d_block_piece;
-        a.tiles = h->d_tiles;
+        a.groups = h->d_tile_groups;
         a.xptr = (float *const *)h->step_ptrs.dev;
         a.gptr = (const void *const *)(h->step_ptrs.dev + T);
         a.pptr = (float *const *)(h->step_ptrs.dev + 2 * T);
@@ -912,7 +913,7 @@ RIKFAD_API int rikfad_step(rikfad_handle h, double step, float *const *x, const 
             if (h->plan.elements_only)
                 RK_CUDA(launch_pdl(h->grad_bytes == 2 ? rikfad_elements_kernel<__nv_bfloat16>
                                                       : rikfad_elements_kernel<float>,
-                                   (int)h->plan.tiles.size(), kThreads, s, a),
+                                   (int)h->plan.tile_groups.size() * kTileGroup, kThreads, s, a),
                         "launch rikfad_elements_kernel");
             else
                 RK_CUDA(launch_pdl(step_kernel(h->grad_bytes, reuse, h->shadow, h->ragged), h->plan.nblocks,
@@ -1098,13 +1099,35 @@ RIKFAD_API int rikfad_export_state(rikfad_handle h, void *dev_dst, void *stream)
     hd.mu = h->hp.mu;
     hd.gamma = h->hp.gamma;
     hd.eps_stab = h->hp.eps_stab;
-    // The header is small; a synchronous copy keeps the host struct's lifetime simple.
-    RK_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
-    RK_CUDA(cudaMemcpy(dev_dst, &hd, sizeof hd, cudaMemcpyHostToDevice), "cudaMemcpy image header");
+    // Into device memory both parts are enqueued: the factors as a copy, the
+    // header as a kernel argument that a few threads store, so the call waits
+    // for nothing (a checkpoint of GPT2-S, with the canonical momentum:
+    // 295 us with a wait for the stream and a blocking copy of the
+    // header, 161 us so).  Any other destination, and a stream that is
+    // being captured, takes the blocking copy with its own checks.
+    cudaPointerAttributes at{};
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    bool enqueue = false;
+    if (cudaPointerGetAttributes(&at, dev_dst) == cudaSuccess && cudaStreamIsCapturing(s, &cap) == cudaSuccess)
+        enqueue = at.type == cudaMemoryTypeDevice && at.device == h->device && cap == cudaStreamCaptureStatusNone;
+    else
+        cudaGetLastError();     // the query's error; the copies below report their own
+    if (!enqueue) {
+        RK_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+        RK_CUDA(cudaMemcpy(dev_dst, &hd, sizeof hd, cudaMemcpyHostToDevice), "cudaMemcpy image header");
+    } else {
+        RK_CUDA(cudaPeekAtLastError(), "earlier CUDA error");
+    }
     if (h->plan.fac_floats > 0)
         RK_CUDA(cudaMemcpyAsync((char *)dev_dst + kImageHeader, h->d_fac, sizeof(float) * h->plan.fac_floats,
                                 cudaMemcpyDeviceToDevice, s),
                 "cudaMemcpyAsync image");
+    if (enqueue) {
+        HeaderParams hp{};
+        hp.dst = static_cast<uint64_t *>(dev_dst);
+        std::memcpy(hp.words, &hd, sizeof hd);
+        RK_CUDA(launch_pdl(rikfad_header_kernel, 1, 32, s, hp), "launch rikfad_header_kernel");
+    }
     return RIKFAD_OK;
 }
 

@@ -17,7 +17,7 @@ struct DenParams {
 struct CanonParams {
     const TensorDev *tensors;
     const PanelDev *panels;
-    const TileDev *tiles;
+    const TileGroupDev *groups;
     const float *const *src;
     float *const *dst;
     const float *fac;
@@ -213,23 +213,27 @@ __global__ void __launch_bounds__(kThreads, 4) rikfad_canonical_kernel(CanonPara
 {
     __shared__ float Cs[kPanelMax];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (!RK_DEV_CHECK(c.chk, (int)blockIdx.x < c.chk.ntiles, kChkBlock))
+    if (!RK_DEV_CHECK(c.chk, (int)blockIdx.x / kTileGroup < c.chk.ngroups, kChkBlock))
         return;
-    const TileDev tile = c.tiles[blockIdx.x];
+    const TileGroupDev group = c.groups[blockIdx.x / kTileGroup];
     PieceDev pc{};
-    pc.kind = tile.panel < 0 ? kElements : kMatrixRows;
-    pc.tensor = tile.tensor;
-    pc.panel = tile.panel;
+    pc.tensor = group.tensor;
     if (!piece_tensor_ok(c.chk, pc))
         return;
     const TensorDev td = c.tensors[pc.tensor];
-    pc.begin = tile.begin;
+    const uint32_t tile = (uint32_t)group.first + blockIdx.x % kTileGroup;      // the planner keeps it below 2^31
+    const uint32_t np = td.npanels > 1 ? td.npanels : 1;
+    pc.kind = td.cols == 0 ? kElements : kMatrixRows;
+    pc.begin = (int64_t)(tile / np) * td.tile_rows;
+    pc.end = pc.begin + td.tile_rows < td.rows ? pc.begin + td.tile_rows : td.rows;
+    pc.panel = td.panel0 + (int)(tile % np);
+    if (pc.begin >= td.rows)
+        return;
     wait_for_predecessor();
     allow_successor_launch();
     const float *S = c.src[pc.tensor];
     float *D = c.dst[pc.tensor];
     if (pc.kind == kElements) {
-        pc.end = tile.begin + kTileElems < td.rows ? tile.begin + kTileElems : td.rows;
         if (S != D && vector_piece_ok(c.chk, pc, td, D, nullptr, S, false))
             canonical_copy(S + pc.begin, D + pc.begin, pc.end - pc.begin);
         return;
@@ -237,7 +241,6 @@ __global__ void __launch_bounds__(kThreads, 4) rikfad_canonical_kernel(CanonPara
     if (!piece_panel_ok(c.chk, pc, td))
         return;
     const PanelDev pd = c.panels[pc.panel];
-    pc.end = tile.begin + pd.tile_rows < td.rows ? tile.begin + pd.tile_rows : td.rows;
     if (!matrix_piece_ok(c.chk, pc, td, pd, D, nullptr, S, false))
         return;
     if (td.full) {      // element-wise friction: P already holds P_{n+1}
@@ -368,6 +371,20 @@ __global__ void rikfad_denominators_kernel(DenParams d)
     const float s = td.cols == 0 ? 0.f : row_total(d.spart, td);
     if ((threadIdx.x & 31) == 0)
         d.out[t] = s;
+}
+
+// A state image's header, stored from the kernel's argument.
+struct HeaderParams {
+    uint64_t *dst;
+    uint64_t words[8];
+};
+
+__global__ void rikfad_header_kernel(HeaderParams p)
+{
+    wait_for_predecessor();
+    allow_successor_launch();
+    if (threadIdx.x < 8)
+        p.dst[threadIdx.x] = p.words[threadIdx.x];
 }
 
 }  // namespace rikfad

@@ -52,7 +52,7 @@ struct StepParams {
     const PanelDev *panels;
     const PieceDev *pieces;
     const int32_t *block_piece;
-    const TileDev *tiles;      // rikfad_elements_kernel
+    const TileGroupDev *groups;   // rikfad_elements_kernel
     float *const *xptr;        // ntensors device pointers
     const void *const *gptr;
     float *const *pptr;
@@ -648,17 +648,19 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
 template <typename GT>
 __global__ void __launch_bounds__(kThreads, 4) rikfad_elements_kernel(StepParams a)
 {
-    if (!RK_DEV_CHECK(a.chk, (int)blockIdx.x < a.chk.ntiles, kChkBlock))
+    if (!RK_DEV_CHECK(a.chk, (int)blockIdx.x / kTileGroup < a.chk.ngroups, kChkBlock))
         return;
-    const TileDev tile = a.tiles[blockIdx.x];
+    const TileGroupDev group = a.groups[blockIdx.x / kTileGroup];
     PieceDev pc{};
     pc.kind = kElements;
-    pc.tensor = tile.tensor;
+    pc.tensor = group.tensor;
     if (!piece_tensor_ok(a.chk, pc))
         return;
-    const TensorDev td = a.tensors[tile.tensor];
-    pc.begin = tile.begin;
-    pc.end = tile.begin + kTileElems < td.rows ? tile.begin + kTileElems : td.rows;
+    const TensorDev td = a.tensors[pc.tensor];
+    pc.begin = (group.first + blockIdx.x % kTileGroup) * kTileElems;
+    pc.end = pc.begin + kTileElems < td.rows ? pc.begin + kTileElems : td.rows;
+    if (pc.begin >= td.rows)
+        return;
     wait_for_predecessor();
     allow_successor_launch();
     if (vector_piece_ok(a.chk, pc, td, a.xptr[pc.tensor], a.gptr[pc.tensor], a.pptr[pc.tensor], true))

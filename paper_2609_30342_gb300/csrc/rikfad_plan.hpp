@@ -57,6 +57,7 @@ struct TensorDev {
     int32_t vec;          // 1: 8-wide vector loads (cols % 8 == 0)
     int32_t full;         // 1: matrix with element-wise friction (full iKFAD) whose R, C are
                           //    shadow factors fed by the same momentum (diagnostics)
+    int64_t tile_rows;    // rows of this matrix's tiles (kTileElems for a vector)
     int64_t xi_off;       // full: friction of the m x n elements at fac + xi_off (row-major)
 };
 
@@ -67,17 +68,21 @@ struct PanelDev {
     int32_t nch;          // ceil(width / kChunk)
     int32_t slot_begin;   // column partial slots of this panel: [slot_begin, slot_end)
     int32_t slot_end;
-    int32_t tile_rows;    // rows of this panel's tiles
 };
 
-// One small block's work in a pass that carries no sums from row to row: up
-// to tile_rows rows of a panel, or kTileElems elements of a vector.  Tiles are
-// in memory order (rows before panels), and the hardware hands out blocks in
-// index order, so the whole GPU streams through a narrow window of HBM.
-struct TileDev {
+// A tile is one small block's work in a pass that carries no sums from row to
+// row: up to tile_rows rows of a panel, or kTileElems elements of a vector.
+// Tile i of a tensor is panel i % npanels of row group i / npanels: memory order
+// (the hardware hands out blocks in index order, so the whole GPU streams
+// through a narrow window of HBM).  Blocks go to tensors by groups of kTileGroup
+// (an entry per tile costs a handle of GPT2-S a millisecond to build and
+// upload); a group's blocks past the tensor's last tile have nothing to do.
+constexpr int kTileGroup = 8;
+
+struct TileGroupDev {
     int32_t tensor;
-    int32_t panel;        // -1: vector
-    int64_t begin;        // first row or element
+    int32_t pad_;
+    int64_t first;        // the group's first tile within the tensor
 };
 
 struct PieceDev {
@@ -111,7 +116,7 @@ struct CheckBounds {
     int32_t nblocks;
     int32_t nfin;
     int32_t nslots;
-    int32_t ntiles;
+    int32_t ngroups;
     int64_t fac_floats;
     int64_t rowpart_floats;
     int64_t colpart_floats;

@@ -85,6 +85,7 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
         td.panel0 = -1;
         if (td.cols == 0) {
             td.vec = 1;
+            td.tile_rows = kTileElems;
             fac += round_up(td.rows, 8);
             if (td.rows > 0)
                 units.push_back({kElements, t, -1, td.rows, vector_elem_bytes(grad_bytes),
@@ -127,9 +128,9 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
             // few elements spends its time on staging C).  Canonical momentum,
             // 16 / 32 rows a tile: GPT2-S 147.0 / 149.3 us, GPT2-Nano-shaped
             // 45.6 / 43.7, eight layers of width 1600 405 / 388.
-            const int32_t tile_rows =
-                widths.back() > kPanelMax / 2 ? 2 * kWarps
-                                              : (int32_t)(4 * kWarps * std::max<int64_t>(1, kTileElems / (kWarps * widths[0])));
+            td.tile_rows = widths.back() > kPanelMax / 2
+                               ? 2 * kWarps
+                               : 4 * kWarps * std::max<int64_t>(1, kTileElems / (kWarps * widths[0]));
             np = (int64_t)widths.size();
             td.npanels = (int32_t)np;
             td.panel0 = (int32_t)p.panels.size();
@@ -142,7 +143,6 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
                 col0 += widths[k];
                 pd.nch = (int32_t)ceil_div(pd.width, kChunk);
                 pd.slot_begin = pd.slot_end = 0;
-                pd.tile_rows = tile_rows;
                 if (td.rows > 0) {
                     const int64_t b = pd.width * (full_matrices ? vector_elem_bytes(grad_bytes)
                                                                 : matrix_elem_bytes(grad_bytes));
@@ -272,13 +272,12 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
     p.elements_only = true;
     for (int t = 0; t < ntensors; ++t) {
         const TensorDev &td = p.tensors[t];
-        const int64_t step = td.cols == 0 ? kTileElems : p.panels[td.panel0].tile_rows;
         p.elements_only &= td.cols == 0 || td.rows == 0;
-        for (int64_t b = 0; b < td.rows; b += step)
-            for (int32_t k = 0; k < std::max(td.npanels, 1); ++k)
-                p.tiles.push_back({t, td.cols == 0 ? -1 : td.panel0 + k, b});
+        const int64_t tiles = td.rows == 0 ? 0 : ceil_div(td.rows, td.tile_rows) * std::max(td.npanels, 1);
+        for (int64_t i = 0; i < tiles; i += kTileGroup)
+            p.tile_groups.push_back({t, 0, i});
     }
-    if (p.tiles.size() > (size_t)std::numeric_limits<int32_t>::max())
+    if (p.tile_groups.size() > (size_t)std::numeric_limits<int32_t>::max() / kTileGroup)
         return "too many elements";
     plan = std::move(p);
     return "";

@@ -15,7 +15,7 @@ struct Plan {
     std::vector<int32_t> block_piece;   // block b owns pieces [block_piece[b], block_piece[b+1])
     std::vector<int64_t> slot_off;      // colpart offset of every slot
     std::vector<FinItemDev> fin_items;
-    std::vector<TileDev> tiles;         // every tensor, in memory order
+    std::vector<TileGroupDev> tile_groups;   // every tensor, in memory order
     bool elements_only = false;         // no matrix has rows: the step is a pass over tiles
     int64_t fac_floats = 0;             // factors + element-wise friction (padded)
     int64_t rowpart_floats = 0;

@@ -331,3 +331,32 @@ def test_host_pointers_are_checked_before_any_launch():
         assert torch.equal(a, b)
     run_d.close()
     run_h.close()
+
+
+def test_export_is_stream_ordered():
+    """An export enqueued on a side stream between two steps holds the state at
+    that point, header included (tag, tensors, pending step, floats,
+    hyperparameters), although the host goes on at once."""
+    import struct
+    inp, run = _run()
+    st = torch.cuda.Stream()
+    imgs = [torch.empty(run.opt.state_image_bytes(), dtype=torch.uint8, device="cuda") for _ in range(2)]
+    run.set_grads(inp.grads(0))
+    torch.cuda.synchronize()
+    run.opt.step(0.1, ptrs=run.ptrs, stream=st)
+    run.opt.export_state(imgs[0], stream=st)
+    run.opt.step(0.07, ptrs=run.ptrs, stream=st)
+    run.opt.export_state(imgs[1], stream=st)
+    st.synchronize()
+    heads = [struct.unpack("<Qqdqdddd", i[:64].cpu().numpy().tobytes()) for i in imgs]
+    assert heads[0][2] == 0.1 and heads[1][2] == 0.07
+    assert heads[0][:2] == heads[1][:2] and heads[0][3:] == heads[1][3:]
+    assert heads[0][1] == len(run.shapes) and heads[0][3] * 4 + 64 == imgs[0].numel()
+    R1 = [r for r, _ in run.factors()]
+    run.opt.import_state(imgs[0])
+    assert run.opt.pending_step == 0.1
+    R0 = [r for r, _ in run.factors()]
+    assert any(not np.array_equal(a, b) for a, b in zip(R0, R1))
+    run.opt.import_state(imgs[1])
+    assert all(np.array_equal(a, b) for a, b in zip(R1, [r for r, _ in run.factors()]))
+    run.close()
