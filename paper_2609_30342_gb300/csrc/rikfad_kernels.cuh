@@ -554,7 +554,7 @@ __device__ __forceinline__ void column_partials(const float *red, float *out, in
 // up to 64 columns and 2 up to kPanelMax / 2 columns; every other one takes 1.
 // A ragged panel takes as many as leave every lane its 8 elements: 4 up to 64
 // columns, 2 up to 128.
-__device__ __forceinline__ int rows_per_warp(bool vec, int w)
+__host__ __device__ __forceinline__ int rows_per_warp(bool vec, int w)
 {
     if (!vec)
         return w <= kChunk / 4 ? 4 : w <= kChunk / 2 ? 2 : 1;

@@ -15,11 +15,21 @@
 // All calls share that one array and it keeps the last call's contents.  A
 // call needs nothing in it to start at zero: it writes every partial sum it
 // later reads (the partial sums of R, the row sums, the column partials)
-// before reading them, in three launches ordered on the caller's stream.  Two
-// calls whose kernels overlap on the GPU (different streams, no ordering)
-// race on the array and produce wrong results.
+// before reading them, in two or three launches ordered on the caller's stream
+// and chained by programmatic dependent launch.  Two calls whose kernels overlap
+// on the GPU (different streams, no ordering) race on the array and produce wrong
+// results.
+//
+// Bound by HBM for the streaming pass and by launches around it.  16384 x 768
+// with bf16 gradients (227 MB): 45.4 us a call, against 51.7 with plain launches
+// and a factor filter of 8 warps per 32 columns over all 304 blocks' partials;
+// 40000 x 512, fp32: 73 against 79; 3000 x 1001, fp32: 21 against 55 (single
+// elements batched, see matrix_piece_ragged).  Filtering R_i in the streaming
+// pass, row by row, cost it more than the row sums' way through memory (50.4 and
+// 86.5 us): the store to R orders the next row's load of R behind it.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <string>
@@ -37,6 +47,8 @@ constexpr int kNaMaxBlocks = 304;                // step blocks: 2 per SM of a G
 constexpr int kNaRowGroup = 1024;                // rows per partial sum of R
 constexpr int64_t kNaRsumFloats = kNaMaxRows / kNaRowGroup;     // 64
 constexpr int kNaColsPerItem = 32;               // columns per block of the column finalise
+constexpr int kNaFinThreads = 1024;              // threads of the finalise: 32 warps share the partials
+constexpr int64_t kNaSumRows = 4096;             // up to here every block adds R itself (one launch less)
 constexpr int64_t kNaScratchFloats = kNaRsumFloats + kNaMaxRows + (int64_t)kNaMaxBlocks * kNaMaxCols;
 
 }  // namespace
@@ -56,6 +68,7 @@ struct NoAllocParams {
     int64_t cols;
     int nblocks;
     int vec;
+    int presummed;            // partial sums of R are in the scratch (rows > kNaSumRows)
     float *x;
     const void *g;
     float *p;
@@ -71,6 +84,8 @@ __global__ void __launch_bounds__(kThreads) rikfad_noalloc_rsum_kernel(const flo
     __shared__ float wsum[kWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t r0 = (int64_t)blockIdx.x * kNaRowGroup;
+    wait_for_predecessor();
+    allow_successor_launch();
     float v = 0.f;
     for (int64_t i = r0 + tid; i < rows && i < r0 + kNaRowGroup; i += kThreads)
         v += R[i];
@@ -103,12 +118,34 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS)
     const int b = blockIdx.x;
     const int w = (int)na.cols;
 
-    // 1^T R from the partial sums, in the same fixed order in every warp.
-    const int nrs = (int)((na.rows + kNaRowGroup - 1) / kNaRowGroup);
+    wait_for_predecessor();
+    // 1^T R in a fixed order, the same in every warp and block: from the partial
+    // sums, or up to kNaSumRows rows from R itself.
     float v = 0.f;
-    for (int k = lane; k < nrs; k += 32)
-        v += rsum[k];
-    const float inv = inv_denominator(warp_sum(v), na.eps);
+    if (na.presummed) {
+        const int nrs = (int)((na.rows + kNaRowGroup - 1) / kNaRowGroup);
+        for (int k = lane; k < nrs; k += 32)
+            v += rsum[k];
+        v = warp_sum(v);
+    } else {
+        __shared__ float wsum[kWarps];
+        float t[kNaSumRows / kThreads];
+#pragma unroll
+        for (int k = 0; k < (int)(kNaSumRows / kThreads); ++k)
+            t[k] = tid + k * kThreads < na.rows ? na.R[tid + k * kThreads] : 0.f;
+#pragma unroll
+        for (int k = 0; k < (int)(kNaSumRows / kThreads); ++k)
+            v += t[k];
+        v = warp_sum(v);
+        if (lane == 0)
+            wsum[tid >> 5] = v;
+        __syncthreads();
+        v = 0.f;
+#pragma unroll
+        for (int k = 0; k < kWarps; ++k)
+            v += wsum[k];
+    }
+    const float inv = inv_denominator(v, na.eps);
     for (int c = tid; c < w; c += kThreads)
         Cs[c] = na.C[c];
     for (int i = tid; i < kWarps * kPanelMax; i += kThreads)
@@ -146,52 +183,96 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS)
     pc.kind = kMatrixRows;
     pc.begin = na.rows * b / na.nblocks;
     pc.end = na.rows * (b + 1) / na.nblocks;
-    if (na.vec)
-        matrix_piece_vec<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
-    else
-        matrix_piece_ragged<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
-    __syncthreads();
-    for (int c = tid; c < w; c += kThreads) {
-        float t = 0.f;
-#pragma unroll
-        for (int k = 0; k < kWarps; ++k)
-            t += red[k * kPanelMax + c];
-        colpart[(int64_t)b * w + c] = t;
+    const int rpw = rows_per_warp(na.vec, w);
+    if (na.vec) {
+        if (rpw == 4)
+            matrix_piece_vec<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
+        else if (rpw == 2)
+            matrix_piece_vec<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
+        else
+            matrix_piece_vec<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
+    } else {
+        if (rpw == 4)
+            matrix_piece_ragged<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
+        else if (rpw == 2)
+            matrix_piece_ragged<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
+        else
+            matrix_piece_ragged<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
     }
+    __syncthreads();
+    allow_successor_launch();
+    float *out = colpart + (int64_t)b * w;
+    if (rpw == 4)
+        column_partials<4>(red, out, w);
+    else if (rpw == 2)
+        column_partials<2>(red, out, w);
+    else
+        column_partials<1>(red, out, w);
 }
 
-// The factor filter: blocks [0, nrow) update kThreads rows of R each from the
-// row sums; the others update kNaColsPerItem columns of C each, the 8 warps
-// adding every 8th block's partial and then the warp sums in order.
-__global__ void __launch_bounds__(kThreads) rikfad_noalloc_finalize_kernel(NoAllocParams na,
-                                                                           const float *scratch, int nrow)
+// The factor filter: blocks [0, ncol) update kNaColsPerItem columns of C each,
+// the 32 warps adding every 32nd block's partial (all loads in flight) and then
+// the warp sums by a fixed tree; the others kNaFinThreads rows of R each from the
+// row sums.
+__global__ void __launch_bounds__(kNaFinThreads) rikfad_noalloc_finalize_kernel(NoAllocParams na,
+                                                                              const float *scratch, int ncol)
 {
-    __shared__ float csum[kWarps][32];
+    constexpr int kFinWarps = kNaFinThreads / 32;
+    constexpr int kPart = (kNaMaxBlocks + kFinWarps - 1) / kFinWarps;
+    __shared__ float csum[kFinWarps][32];
     const float *rowsum = scratch + kNaRsumFloats;
     const float *colpart = scratch + kNaRsumFloats + kNaMaxRows;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if ((int)blockIdx.x < nrow) {
-        const int64_t i = (int64_t)blockIdx.x * kThreads + tid;
+    wait_for_predecessor();
+    allow_successor_launch();
+    if ((int)blockIdx.x >= ncol) {
+        const int64_t i = (int64_t)(blockIdx.x - ncol) * kNaFinThreads + tid;
         if (i < na.rows)
             na.R[i] = fmaf(na.gain, rowsum[i], na.decay * na.R[i]);
         return;
     }
-    const int64_t c = (int64_t)(blockIdx.x - nrow) * kNaColsPerItem + lane;
-    float acc = 0.f;
-    if (c < na.cols) {
-#pragma unroll 4
-        for (int k = warp; k < na.nblocks; k += kWarps)
-            acc += colpart[(int64_t)k * na.cols + c];
+    const int64_t c = (int64_t)blockIdx.x * kNaColsPerItem + lane;
+    float t[kPart];
+#pragma unroll
+    for (int k = 0; k < kPart; ++k) {
+        const int b = warp + k * kFinWarps;
+        t[k] = c < na.cols && b < na.nblocks ? colpart[(int64_t)b * na.cols + c] : 0.f;
     }
+    float acc = 0.f;
+#pragma unroll
+    for (int k = 0; k < kPart; ++k)
+        acc += t[k];
     csum[warp][lane] = acc;
     __syncthreads();
     if (warp == 0 && c < na.cols) {
-        float t = 0.f;
+        float s[kFinWarps];
 #pragma unroll
-        for (int k = 0; k < kWarps; ++k)
-            t += csum[k][lane];
-        na.C[c] = fmaf(na.gain, t, na.decay * na.C[c]);
+        for (int k = 0; k < kFinWarps; ++k)
+            s[k] = csum[k][lane];
+#pragma unroll
+        for (int o = kFinWarps / 2; o > 0; o /= 2)
+#pragma unroll
+            for (int k = 0; k < o; ++k)
+                s[k] += s[k + o];
+        na.C[c] = fmaf(na.gain, s[0], na.decay * na.C[c]);
     }
+}
+
+// A launch that may begin while its predecessor in the stream finishes (each
+// kernel waits before it touches data).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), int nblocks, int nthreads, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nblocks);
+    cfg.blockDim = dim3((unsigned)nthreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 // Device address of the scratch array, looked up once per device.
@@ -262,7 +343,10 @@ extern "C" RIKFAD_API int rikfad_step_matrix_noalloc(int64_t rows, int64_t cols,
     NoAllocParams na{};
     na.rows = rows;
     na.cols = cols;
-    na.nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(kNaMaxBlocks, rows));
+    // A block has at least a row for each of its warps' lane groups.
+    const int64_t per_block = (int64_t)kWarps * rows_per_warp(vec, (int)cols);
+    na.nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(kNaMaxBlocks, (rows + per_block - 1) / per_block));
+    na.presummed = rows > kNaSumRows;
     na.vec = vec;
     na.x = x;
     na.g = grad;
@@ -277,26 +361,22 @@ extern "C" RIKFAD_API int rikfad_step_matrix_noalloc(int64_t rows, int64_t cols,
     na.gain = std::isinf(hp->mu) ? 0.f : (float)(-std::expm1(-hp->alpha * step) / (hp->mu * hp->alpha));
     na.eps = (float)hp->eps_stab;
     const bool reuse = step == pending_step;
-    // Three launches on the caller's stream: partial sums of R, the
+    // On the caller's stream: partial sums of R (more than kNaSumRows rows), the
     // streaming pass, the factor filter.
     const int nrs = (int)((rows + kNaRowGroup - 1) / kNaRowGroup);
-    if (nrs > 0)
-        rikfad_noalloc_rsum_kernel<<<nrs, kThreads, 0, s>>>(R, rows, scratch);
-    if (grad_dtype == RIKFAD_GRAD_BF16) {
-        if (reuse)
-            rikfad_noalloc_step_kernel<__nv_bfloat16, true><<<na.nblocks, kThreads, 0, s>>>(na, scratch);
-        else
-            rikfad_noalloc_step_kernel<__nv_bfloat16, false><<<na.nblocks, kThreads, 0, s>>>(na, scratch);
-    } else {
-        if (reuse)
-            rikfad_noalloc_step_kernel<float, true><<<na.nblocks, kThreads, 0, s>>>(na, scratch);
-        else
-            rikfad_noalloc_step_kernel<float, false><<<na.nblocks, kThreads, 0, s>>>(na, scratch);
-    }
-    const int nrow = (int)((rows + kThreads - 1) / kThreads);
+    cudaError_t e = cudaSuccess;
+    if (na.presummed)
+        e = launch_chained(rikfad_noalloc_rsum_kernel, nrs, kThreads, s, (const float *)R, rows, scratch);
+    auto pass = grad_dtype == RIKFAD_GRAD_BF16
+                    ? (reuse ? rikfad_noalloc_step_kernel<__nv_bfloat16, true>
+                             : rikfad_noalloc_step_kernel<__nv_bfloat16, false>)
+                    : (reuse ? rikfad_noalloc_step_kernel<float, true> : rikfad_noalloc_step_kernel<float, false>);
+    if (e == cudaSuccess)
+        e = launch_chained(pass, na.nblocks, kThreads, s, na, scratch);
+    const int nrow = (int)((rows + kNaFinThreads - 1) / kNaFinThreads);
     const int ncol = (int)((cols + kNaColsPerItem - 1) / kNaColsPerItem);
-    rikfad_noalloc_finalize_kernel<<<nrow + ncol, kThreads, 0, s>>>(na, scratch, nrow);
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = launch_chained(rikfad_noalloc_finalize_kernel, ncol + nrow, kNaFinThreads, s, na, (const float *)scratch, ncol);
     if (e != cudaSuccess)
         return na_fail(RIKFAD_ERR_CUDA, cudaGetErrorString(e));
     return RIKFAD_OK;

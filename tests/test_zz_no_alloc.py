@@ -139,3 +139,42 @@ def test_noalloc_binding_checks_buffers():
     rikfad.step_matrix_noalloc(rows, cols, 0.1, 0.0, 0.5, 1.0, 0.0, 1e-8, "f32", ok["x"], ok["grad"],
                                ok["p"], ok["R"], ok["C"])
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("rows,cols,grad", [(1, 1, "f32"), (7, 8, "bf16"), (33, 64, "f32"), (4096, 40, "bf16"),
+                                            (4097, 40, "bf16"), (2433, 127, "f32"), (9729, 65, "bf16"),
+                                            (1025, 33, "bf16"), (5000, 384, "f32"), (4095, 1023, "bf16")])
+def test_noalloc_at_the_edges_of_its_launches(rows, cols, grad):
+    """Row counts around the two ways to 1^T R (4096) and around one row per
+    lane group of 304 blocks, widths of every rows-per-warp path: three calls
+    against the oracle from the call before's state, X and P^(1) within 1e-5 or
+    the per-element bound, R and C within 1e-5 (their sums' depths are below
+    64 additions a level, 1e-5 is 168 roundings of positive terms)."""
+    pkg_build.build()
+    dev, X0, P0, G = _inputs(rows, cols, grad)
+    x, p = X0.to(dev), P0.to(dev)
+    R = torch.rand(rows, device=dev, generator=torch.Generator(device=dev).manual_seed(1))
+    C = torch.rand(cols, device=dev, generator=torch.Generator(device=dev).manual_seed(2))
+    hp = oracle.HParams(**HP)
+    pending = 0.0
+    for k, h in enumerate(STEPS):
+        Xo, Ro, Co = (t.double().cpu().numpy() for t in (x, R, C))
+        Xo = np.ascontiguousarray(Xo)
+        Ps = p.double().cpu().numpy()
+        xi = np.outer(Ro, Co) / (Ro.sum() + hp.eps_stab)
+        Po = np.ascontiguousarray(Ps * np.exp(-0.5 * pending * xi) * np.exp(-hp.gamma * pending))
+        P1o = np.empty((rows, cols))
+        X00, P00 = Xo.copy(), Po.copy()
+        g = np.ascontiguousarray(G[k].double().numpy())
+        oracle.step_matrix(Xo, Po, Ro, Co, g, h, hp, P1=P1o)
+        rikfad.step_matrix_noalloc(rows, cols, h, pending, HP["alpha"], HP["mu"], HP["gamma"], HP["eps_stab"],
+                                   grad, x, G[k].to(dev), p, R, C)
+        torch.cuda.synchronize()
+        pending = h
+        compare("R", R.double().cpu().numpy(), Ro, 1e-5, 0.0)
+        compare("C", C.double().cpu().numpy(), Co, 1e-5, 0.0)
+        # X, P^(1): relative, or a rounding of the larger terms where they cancel
+        for name, got, want, terms in (("X", x, Xo, np.abs(X00) + 2 * np.abs(Xo - X00)),
+                                       ("P", p, P1o, np.abs(P00) + 2 * h * np.abs(g))):
+            err = np.abs(got.double().cpu().numpy() - want)
+            assert np.all(err <= np.maximum(1e-5 * np.abs(want), 8 * 2.0 ** -24 * terms)), (name, k, err.max())
