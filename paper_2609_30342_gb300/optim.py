@@ -13,9 +13,15 @@ device (autograd gives a float32 parameter a float32 gradient; bfloat16
 gradients are for the pointer API, ``rikfad.RIKFAD``).  A parameter without a
 gradient at a step takes a zero gradient, since the handle steps a fixed list.
 """
+from operator import attrgetter, is_, itemgetter
+
 import torch
 
 from . import rikfad
+
+# The marshalling below runs over every parameter at every step: C-level maps
+# of these keep it within a small model's kernel time.
+_grad, _dtype, _momentum = attrgetter("grad"), attrgetter("dtype"), itemgetter("momentum")
 
 
 class RIKFADOptimizer(torch.optim.Optimizer):
@@ -33,7 +39,7 @@ class RIKFADOptimizer(torch.optim.Optimizer):
     def _group_handle(self, i, group):
         params = group["params"]
         entry = self._groups.get(i)
-        if entry is not None and len(entry[1]) == len(params) and all(a is b for a, b in zip(entry[1], params)):
+        if entry is not None and len(entry[1]) == len(params) and all(map(is_, entry[1], params)):
             return entry
         if entry is not None:
             entry[0].close()
@@ -49,13 +55,14 @@ class RIKFADOptimizer(torch.optim.Optimizer):
         return entry
 
     def _momenta(self, params):
-        out = []
-        for p in params:
-            st = self.state[p]
-            if "momentum" not in st:
-                st["momentum"] = torch.zeros_like(p)
-            out.append(st["momentum"])
-        return out
+        state = self.state
+        try:
+            return list(map(_momentum, map(state.__getitem__, params)))
+        except KeyError:        # a parameter's first step
+            for p in params:
+                if "momentum" not in state[p]:
+                    state[p]["momentum"] = torch.zeros_like(p)
+        return [state[p]["momentum"] for p in params]
 
     @torch.no_grad()
     def step(self, closure=None):
@@ -67,12 +74,9 @@ class RIKFADOptimizer(torch.optim.Optimizer):
             if not group["params"]:
                 continue
             handle, params, zeros = self._group_handle(i, group)
-            grads = []
-            for p, z in zip(params, zeros):
-                g = p.grad
-                if g is not None and not (g.dtype == torch.float32 and g.is_contiguous()):
-                    raise ValueError("gradients must be contiguous float32 tensors")
-                grads.append(z if g is None else g)
+            grads = [z if g is None else g for g, z in zip(map(_grad, params), zeros)]
+            if not (all(map(torch.Tensor.is_contiguous, grads)) and set(map(_dtype, grads)) == {torch.float32}):
+                raise ValueError("gradients must be contiguous float32 tensors")
             handle.step(group["lr"], params, grads, self._momenta(params),
                         stream=torch.cuda.current_stream(params[0].device))
         return loss
