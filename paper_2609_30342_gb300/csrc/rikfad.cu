@@ -1275,21 +1275,20 @@ RIKFAD_API int rikfad_friction_diagnostics(rikfad_handle h, int t, int max_iters
     d.v2part = h->d_diag_v2part;
     d.st = h->d_diag_state;
     d.host = h->h_diag_state_dev;
-    // Iterations are enqueued kDiagIters at a time; after convergence the
-    // kernels left in the queue return at once.
+    // kDiagIters iterations are enqueued at once, then two more whenever the
+    // host finds them not enough; kernels queued past convergence return at once.
     const bool vec = n % 4 == 0 && n <= kDiagStageCols;
     const size_t smem = n <= kDiagStageCols ? (size_t)((n + 3) / 4 * 8) * sizeof(float) : 0;
     const DiagState &st = *h->h_diag_state;
-    RK_CUDA(cudaMemsetAsync(h->d_diag_state, 0, sizeof(DiagState), s), "cudaMemsetAsync");
     for (int it = 0; it < max_iters;) {
-        const int64_t stop = std::min<int64_t>(max_iters, (int64_t)it + kDiagIters);
+        const int64_t stop = std::min<int64_t>(max_iters, (int64_t)it + (it == 0 ? kDiagIters : 2));
         for (; it < stop; ++it) {
             d.parity = it & 1;
             d.last = it + 1 == stop;
             auto rows = it == 0 ? (vec ? rikfad_diag_rows_kernel<true, true> : rikfad_diag_rows_kernel<true, false>)
                                 : (vec ? rikfad_diag_rows_kernel<false, true> : rikfad_diag_rows_kernel<false, false>);
             RK_CUDA(launch_pdl(rows, d.nblk, kThreads, s, d, smem), "launch rikfad_diag_rows_kernel");
-            RK_CUDA(launch_pdl(rikfad_diag_cols_kernel, d.ncb, kThreads, s, d), "launch rikfad_diag_cols_kernel");
+            RK_CUDA(launch_pdl(rikfad_diag_cols_kernel, d.ncb, diag_col_threads(d.nblk), s, d), "launch rikfad_diag_cols_kernel");
         }
         RK_CUDA(cudaStreamSynchronize(s), "power iteration");
         if (st.done)

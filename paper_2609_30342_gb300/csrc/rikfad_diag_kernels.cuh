@@ -27,7 +27,7 @@
 // per-block partial sums.  Bound by launch and L2 latency for a layer's 2 to 10
 // MB, by the one read of xi for larger matrices.  Measured on GB300, six calls
 // for the layers of a GPT2-S block: 3800 to 7400 us (by seed) with four kernels an
-// iteration in a captured graph and the plain quotient, 354 us so.
+// iteration iteration in a captured graph and the plain quotient, 346 us so.
 #pragma once
 #include <algorithm>
 
@@ -39,7 +39,11 @@ constexpr int kDiagMaxBlocks = 456;      // row blocks: 3 per SM of a GB300
 constexpr int kDiagStageCols = 4096;     // widest xi whose iterate and sums are staged in shared memory
 constexpr int kDiagMaxColBlocks = 512;   // column blocks (each adds all of their sums of v^2)
 constexpr int64_t kDiagMaxPartials = 1 << 24;   // floats of row-block partials (more only at 32 rows a block)
-constexpr int kDiagIters = 4;            // iterations enqueued before the host looks
+// Threads of the column kernel, whose warps share the partials of 32 columns:
+// 1024 beyond 128 row blocks (768 x 768, 192 of them: 51 us a call against 59 with
+// 256), else 256 (64 x 4096, 64 of them: 64 against 69 with 1024).
+inline int diag_col_threads(int nblk) { return nblk > 128 ? 1024 : 256; }
+constexpr int kDiagIters = 4;            // iterations enqueued before the host first looks
 
 // State of one power iteration, in device memory; the record the host reads
 // is a copy in mapped host memory.
@@ -189,7 +193,9 @@ __global__ void __launch_bounds__(kThreads, FIRST && VEC ? 2 : 3) rikfad_diag_ro
             wacc[j] = 0.f;
     __syncthreads();
     auto v_at = [&](int64_t j) { return FIRST && !staged ? first_v(v[j]) : v[j]; };
-    if (FIRST && blockIdx.x == 0) {     // ||v||^2 of the first iterate
+    if (FIRST && blockIdx.x == 0) {     // a cleared state; ||v||^2 of the first iterate
+        if (tid == 0)
+            *d.st = DiagState{};
         double a = 0.0;
         for (int64_t j = tid; j < n; j += kThreads) {
             const double t = (double)v_at(j);
@@ -385,15 +391,16 @@ __global__ void __launch_bounds__(kThreads, FIRST && VEC ? 2 : 3) rikfad_diag_ro
 
 // Column kernel: cpb columns a block, 32 at a time.  The next iterate v =
 // (xi^T u) ||v||^2 / ||u||^2 (whose length stays near the last one's and equals
-// it once converged): warp k adds the row blocks k, k + 8, ... in order, then
-// warp 0 the eight warp sums; its squares go to the other half of v2part.
+// it once converged): warp k of W adds the row blocks k, k + W, ... in order, then
+// warp 0 the W warp sums; its squares go to the other half of v2part.
 // Block 0 forms the quotient and tests convergence: |sigma^2 - previous| <= tol
 // sigma^2 from the second iteration on, or max_iters, or nothing left to
 // iterate on.
-__global__ void __launch_bounds__(kThreads) rikfad_diag_cols_kernel(DiagParams d)
+__global__ void __launch_bounds__(1024) rikfad_diag_cols_kernel(DiagParams d)
 {
     constexpr int kU = 8;
-    __shared__ float part[kWarps][32];
+    __shared__ float part[32][32];
+    const int nwarps = blockDim.x >> 5;
     __shared__ double tot[4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n = d.td.cols;
@@ -418,11 +425,11 @@ __global__ void __launch_bounds__(kThreads) rikfad_diag_cols_kernel(DiagParams d
         const int64_t j = (int64_t)blockIdx.x * d.cpb + c0 + lane;
         float acc = 0.f;
         if (j < n) {
-            for (int g0 = warp; g0 < d.nblk; g0 += kWarps * kU) {
+            for (int g0 = warp; g0 < d.nblk; g0 += nwarps * kU) {
                 float t[kU];
 #pragma unroll
                 for (int k = 0; k < kU; ++k) {
-                    const int g = g0 + k * kWarps;
+                    const int g = g0 + k * nwarps;
                     t[k] = g < d.nblk ? d.wpart[(int64_t)g * n + j] : 0.f;
                 }
 #pragma unroll
@@ -435,8 +442,8 @@ __global__ void __launch_bounds__(kThreads) rikfad_diag_cols_kernel(DiagParams d
         __syncthreads();
         if (warp == 0 && j < n) {
             float sum = 0.f;
-#pragma unroll
-            for (int k = 0; k < kWarps; ++k)
+#pragma unroll 8
+            for (int k = 0; k < nwarps; ++k)
                 sum += part[k][lane];
             const float vn = tot[0] > 0.0 ? (float)((double)sum * (tot[1] / tot[0])) : 0.f;
             d.v[j] = vn;
