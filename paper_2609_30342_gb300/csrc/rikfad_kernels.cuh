@@ -189,7 +189,7 @@ __device__ __forceinline__ float matrix_element(float &x, float p_hat, float g, 
 
 // ACCUM: add each row's squares into the warp's column buffer (several rows
 // per warp); otherwise store them (one row per warp, buffer not cleared).
-// RPW rows per warp (1, 2 or 4; panels of at most kPanelMax / RPW columns):
+// RPW rows per warp (1, 2, 4 or 8; panels of at most kPanelMax / RPW columns):
 // each of the warp's RPW lane groups takes its own row, 256 / RPW columns per
 // chunk, so a panel whose width is not a multiple of 256 still loads 256
 // columns per warp and round trip; group h accumulates its columns at
@@ -439,12 +439,20 @@ __device__ __forceinline__ float full_element(float &x, float &p, float &xi, flo
     return p1 * p1;
 }
 
-template <typename GT, bool RAGGED>
+//
+// Rows per warp and loads in flight as matrix_piece_vec (VEC) and
+// matrix_piece_ragged: one row per warp left most lanes of a narrow panel idle
+// (bf16 gradients, share of the 6.8 TB/s floor: width 24 0.20 -> 0.76, 64 0.49 ->
+// 0.88, 640 0.71 -> 0.87, 9000 0.39 -> 0.81).
+template <typename GT, bool VEC, int RPW>
 __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const PieceDev &pc,
                                                   const TensorDev &td, const PanelDev &pd,
                                                   float *red)
 {
+    constexpr int kRowLanes = 32 / RPW;                 // lanes per row
+    constexpr int kU = 8;                               // ragged: elements per lane and pass
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rl = lane & (kRowLanes - 1), half = lane / kRowLanes;
     const int64_t n = td.cols;
     const int w = pd.width;
     float *X = a.xptr[pc.tensor];
@@ -452,49 +460,46 @@ __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const Pie
     float *P = a.pptr[pc.tensor];
     float *XI = a.fac + td.xi_off;
     float *rowpart = a.rowpart + td.rowpart_off + (int64_t)(pc.panel - td.panel0) * td.rows;
-    float *myred = red + warp * kPanelMax;
-    for (int64_t row = pc.begin + warp; row < pc.end; row += kWarps) {
+    float *myred = red + warp * kPanelMax + half * (kPanelMax / RPW);
+    for (int64_t r0 = pc.begin + RPW * warp; r0 < pc.end; r0 += RPW * kWarps) {
+        const int64_t row = r0 + half;
+        const bool live = RPW == 1 || row < pc.end;
         const int64_t base = row * n + pd.col0;
+        const int wl = live ? w : 0;
         float racc = 0.f;
-        if (!RAGGED || td.vec) {
+        if (VEC) {
 #pragma unroll 1
-            for (int ch = 0; ch < pd.nch; ++ch) {
-                const int c = ch * kChunk + lane * 8;
-                if (c < w) {
-                    Grad8<GT> gv;
-                    gv.load(G + base + c);
-                    float x[8], p[8], xi[8];
-                    load8(X + base + c, x);
-                    load8(P + base + c, p);
-                    load8(XI + base + c, xi);
-                    float q[8];
+            for (int c = rl * 8; c < wl; c += kRowLanes * 8) {
+                Grad8<GT> gv;
+                gv.load(G + base + c);
+                float x[8], p[8], xi[8];
+                load8(X + base + c, x);
+                load8(P + base + c, p);
+                load8(XI + base + c, xi);
+                float q[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        q[e] = full_element(x[e], p[e], xi[e], gv.get(e), a);
-                        racc += q[e];
-                    }
-                    store8(X + base + c, x);
-                    store8(P + base + c, p);
-                    store8(XI + base + c, xi);
-                    float4 *r4 = reinterpret_cast<float4 *>(myred + c);
-                    float4 r0 = r4[0], r1 = r4[1];
-                    r0.x += q[0]; r0.y += q[1]; r0.z += q[2]; r0.w += q[3];
-                    r1.x += q[4]; r1.y += q[5]; r1.z += q[6]; r1.w += q[7];
-                    r4[0] = r0;
-                    r4[1] = r1;
+                for (int e = 0; e < 8; ++e) {
+                    q[e] = full_element(x[e], p[e], xi[e], gv.get(e), a);
+                    racc += q[e];
                 }
+                store8(X + base + c, x);
+                store8(P + base + c, p);
+                store8(XI + base + c, xi);
+                float4 *r4 = reinterpret_cast<float4 *>(myred + c);
+                float4 r0 = r4[0], r1 = r4[1];
+                r0.x += q[0]; r0.y += q[1]; r0.z += q[2]; r0.w += q[3];
+                r1.x += q[4]; r1.y += q[5]; r1.z += q[6]; r1.w += q[7];
+                r4[0] = r0;
+                r4[1] = r1;
             }
         } else {
-            // Rows at any element address: 256 columns' loads before any
-            // arithmetic, as matrix_piece_ragged.
-            constexpr int kU = 8;
 #pragma unroll 1
-            for (int c0 = lane; c0 < w; c0 += 32 * kU) {
+            for (int c0 = rl; c0 < wl; c0 += kRowLanes * kU) {
                 float x[kU], p[kU], xi[kU], g[kU];
 #pragma unroll
                 for (int u = 0; u < kU; ++u)
-                    if (c0 + 32 * u < w) {
-                        const int64_t i = base + c0 + 32 * u;
+                    if (c0 + kRowLanes * u < w) {
+                        const int64_t i = base + c0 + kRowLanes * u;
                         g[u] = grad_at(G, i);
                         x[u] = __ldcs(X + i);
                         p[u] = __ldcs(P + i);
@@ -502,7 +507,7 @@ __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const Pie
                     }
 #pragma unroll
                 for (int u = 0; u < kU; ++u) {
-                    const int c = c0 + 32 * u;
+                    const int c = c0 + kRowLanes * u;
                     if (c < w) {
                         const float q = full_element(x[u], p[u], xi[u], g[u], a);
                         __stcs(X + base + c, x[u]);
@@ -514,8 +519,10 @@ __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const Pie
                 }
             }
         }
-        racc = warp_sum(racc);
-        if (lane == 0)
+#pragma unroll
+        for (int o = kRowLanes / 2; o > 0; o >>= 1)
+            racc += __shfl_xor_sync(0xffffffffu, racc, o);
+        if (live && rl == 0)
             rowpart[row] = racc;
     }
 }
@@ -549,19 +556,23 @@ __device__ __forceinline__ void column_partials(const float *red, float *out, in
     }
 }
 
-// Rows per warp (RPW of matrix_piece_vec and matrix_piece_ragged).  An 8-wide
-// panel that is not a whole number of 256-column chunks takes 4 rows per warp
-// up to 64 columns and 2 up to kPanelMax / 2 columns; every other one takes 1.
-// A ragged panel takes as many as leave every lane its 8 elements: 4 up to 64
-// columns, 2 up to 128.
+// Rows per warp (RPW of the row loops).  An 8-wide panel that is not a whole
+// number of 256-column chunks takes 8 rows per warp up to 32 columns, 4 up to 64
+// and 2 up to kPanelMax / 2 columns; every other one takes 1.  A ragged panel
+// takes as many as leave every lane its 8 elements: 8, 4, 2 up to 32, 64, 128.
+// 40 M elements of width 24, bf16: 4 rows per warp 0.43 of the 6.8 TB/s floor, 8
+// rows 0.64.
 __host__ __device__ __forceinline__ int rows_per_warp(bool vec, int w)
 {
-    if (!vec)
-        return w <= kChunk / 4 ? 4 : w <= kChunk / 2 ? 2 : 1;
-    if (w % kChunk == 0 || w > kPanelMax / 2)
+    if (vec ? (w % kChunk == 0 || w > kPanelMax / 2) : w > kChunk / 2)
         return 1;
-    return w <= kChunk / 4 ? 4 : 2;
+    return w <= kChunk / 8 ? 8 : w <= kChunk / 4 ? 4 : 2;
 }
+
+template <int N>
+struct RowsPerWarp {
+    static constexpr int value = N;
+};
 
 template <typename GT, bool REUSE, bool SHADOW = false, bool RAGGED = false>
 __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_kernel(StepParams a)
@@ -604,33 +615,36 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
             red[i] = 0.f;
         const float inv = inv_denominator(row_total(a.spart, td), a.eps);
         __syncthreads();
-        const int rpw = SHADOW ? 1 : rows_per_warp(!RAGGED || td.vec, w);
-        if (SHADOW) {
-            matrix_piece_full<GT, RAGGED>(a, pc, td, pd, red);
-        } else if (!RAGGED || td.vec) {
-            if (rpw == 4)
-                matrix_piece_vec<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
-            else if (rpw == 2)
-                matrix_piece_vec<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
-            else
-                matrix_piece_vec<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
-        } else {
-            if (rpw == 4)
-                matrix_piece_ragged<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
-            else if (rpw == 2)
-                matrix_piece_ragged<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
-            else
-                matrix_piece_ragged<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
-        }
-        __syncthreads();
-        // Column partial sums of this piece, warps (and their lane groups) added in order.
-        float *out = a.colpart + pc.colpart_off;
-        if (rpw == 1)
-            column_partials<1>(red, out, w);
+        // The RAGGED instantiations carry fewer row loops (1, 2 and 4 rows per
+        // warp; 1 with SHADOW): with more of them the compiler spills inside the
+        // loops (40 M elements, bf16, width 500: 182 us with all, 141 so; as
+        // functions of their own 197).
+        const int rpw = SHADOW && RAGGED ? 1 : rows_per_warp(!RAGGED || td.vec, w);
+        // One call of the piece's path for its rows per warp.
+        auto piece = [&](auto n) {
+            constexpr int N = decltype(n)::value;
+            if (SHADOW) {
+                if (!RAGGED || td.vec)
+                    matrix_piece_full<GT, true, N>(a, pc, td, pd, red);
+                else
+                    matrix_piece_full<GT, false, N>(a, pc, td, pd, red);
+            } else if (!RAGGED || td.vec) {
+                matrix_piece_vec<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv);
+            } else {
+                matrix_piece_ragged<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv);
+            }
+            __syncthreads();
+            // Column partial sums of this piece, warps (and their lane groups) added in order.
+            column_partials<N>(red, a.colpart + pc.colpart_off, w);
+        };
+        if ((SHADOW && RAGGED) || rpw == 1)
+            piece(RowsPerWarp<1>());
         else if (rpw == 2)
-            column_partials<2>(red, out, w);
+            piece(RowsPerWarp<2>());
+        else if (RAGGED || rpw == 4)
+            piece(RowsPerWarp<4>());
         else
-            column_partials<4>(red, out, w);
+            piece(RowsPerWarp<8>());
         __syncthreads();
     }
 }

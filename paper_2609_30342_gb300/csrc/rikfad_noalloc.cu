@@ -184,30 +184,24 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS)
     pc.begin = na.rows * b / na.nblocks;
     pc.end = na.rows * (b + 1) / na.nblocks;
     const int rpw = rows_per_warp(na.vec, w);
-    if (na.vec) {
-        if (rpw == 4)
-            matrix_piece_vec<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
-        else if (rpw == 2)
-            matrix_piece_vec<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
+    auto piece = [&](auto n) {
+        constexpr int N = decltype(n)::value;
+        if (na.vec)
+            matrix_piece_vec<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv);
         else
-            matrix_piece_vec<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
-    } else {
-        if (rpw == 4)
-            matrix_piece_ragged<GT, REUSE, true, 4>(a, pc, td, pd, Cs, red, inv);
-        else if (rpw == 2)
-            matrix_piece_ragged<GT, REUSE, true, 2>(a, pc, td, pd, Cs, red, inv);
-        else
-            matrix_piece_ragged<GT, REUSE>(a, pc, td, pd, Cs, red, inv);
-    }
-    __syncthreads();
-    allow_successor_launch();
-    float *out = colpart + (int64_t)b * w;
-    if (rpw == 4)
-        column_partials<4>(red, out, w);
+            matrix_piece_ragged<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv);
+        __syncthreads();
+        allow_successor_launch();
+        column_partials<N>(red, colpart + (int64_t)b * w, w);
+    };
+    if (rpw == 1)
+        piece(RowsPerWarp<1>());
     else if (rpw == 2)
-        column_partials<2>(red, out, w);
+        piece(RowsPerWarp<2>());
+    else if (rpw == 4)
+        piece(RowsPerWarp<4>());
     else
-        column_partials<1>(red, out, w);
+        piece(RowsPerWarp<8>());
 }
 
 // The factor filter: blocks [0, ncol) update kNaColsPerItem columns of C each,

@@ -80,3 +80,30 @@ def test_ragged_shadow_steps_match_oracle(grad_bf16):
         seeded.step(g, h)
         _compare(run, seeded, 1e-5, "reseeded step%d " % (k + 1))
     run.close()
+
+
+@pytest.mark.parametrize("method", ["rikfad", "ikfad_shadow"])
+@pytest.mark.parametrize("grad_bf16", [True, False])
+def test_narrow_panels_match_oracle(method, grad_bf16):
+    """8-wide panels of every number of rows per warp (8, 4, 2, 1 up to 32, 64,
+    512 and more columns), with row counts that leave lane groups idle, and
+    matrices whose last panel is narrow: from the GPU's own state at 1e-5."""
+    widths = [8, 16, 24, 32, 40, 64, 72, 128, 200, 256, 384, 512, 520, 1096, 1376, 1600]
+    shapes = [(r, w) for w, r in zip(widths, [129, 65, 63, 9, 33, 31, 17, 15, 7, 9, 13, 3, 5, 9, 7, 18])]
+    inp = workloads.ModelInputs(shapes, seed=63, g_std=1e-2, grad_bf16=grad_bf16)
+    run = DeviceRun(shapes, SHADOW_HP, grad_bf16, inp.X, inp.P, method=method)
+    for k, h in enumerate((0.1, 0.1, 0.05)):
+        g = inp.grads(k)
+        if method == "rikfad":
+            seeded = Tracked.from_gpu(run)
+        else:
+            seeded = ShadowRef(shapes, *_gpu_state(run))
+        run.set_grads(g)
+        run.step(h)
+        if method == "rikfad":
+            seeded.step(g, h, SHADOW_HP, run.factors())
+            seeded.check(run, 1e-5, "step%d" % (k + 1))
+        else:
+            seeded.step(g, h)
+            _compare(run, seeded, 1e-5, "step%d " % (k + 1))
+    run.close()
