@@ -148,14 +148,15 @@ def _ptr(t):
 
 def _ptr_array(tensors):
     # 64-bit integers laid out as the C array, viewed by ctypes: a list of 100
-    # tensors packs in a quarter of the time of one c_void_p per entry.
+    # tensors packs in a quarter of the time of one c_void_p per entry, a short
+    # one in more.
+    if len(tensors) <= 8:
+        return (ctypes.c_void_p * max(len(tensors), 1))(*[_ptr(t) for t in tensors])
     import torch
     try:
         ptrs = array.array("Q", map(torch.Tensor.data_ptr, tensors))
     except TypeError:                   # integers, None or other objects among them
         ptrs = array.array("Q", [_ptr(t) or 0 for t in tensors])
-    if not ptrs:
-        ptrs.append(0)
     return (ctypes.c_void_p * len(ptrs)).from_buffer(ptrs)
 
 
