@@ -145,6 +145,7 @@ struct rikfad_handle_s {
     bool pageable_ok = false;       // the device reads pageable host memory (host page tables)
     int ntensors = 0;
     int grad_bytes = 4;
+    size_t wide_smem = 0;           // dynamic shared memory of a step with bands (0: none)
     bool ragged = false;            // a matrix has rows that are not 8-aligned
     rikfad_hparams hp{};
     Plan plan;
@@ -392,6 +393,7 @@ using StepKernel = void (*)(StepParams);
 
 // The step kernel's instantiation for a handle's matrices.  Full-friction
 // matrices (shadow) have no pending factor, so reuse never applies to them.
+// `wide`: the list has bands (never with shadow or ragged).
 template <typename GT, bool RAGGED>
 StepKernel step_kernel(bool reuse, bool shadow)
 {
@@ -400,12 +402,28 @@ StepKernel step_kernel(bool reuse, bool shadow)
     return reuse ? rikfad_step_kernel<GT, true, false, RAGGED> : rikfad_step_kernel<GT, false, false, RAGGED>;
 }
 
-StepKernel step_kernel(int grad_bytes, bool reuse, bool shadow, bool ragged)
+template <typename GT>
+StepKernel step_kernel(bool reuse, bool shadow, bool ragged, bool wide)
 {
-    if (grad_bytes == 2)
-        return ragged ? step_kernel<__nv_bfloat16, true>(reuse, shadow)
-                      : step_kernel<__nv_bfloat16, false>(reuse, shadow);
-    return ragged ? step_kernel<float, true>(reuse, shadow) : step_kernel<float, false>(reuse, shadow);
+    if (wide)
+        return reuse ? rikfad_step_kernel<GT, true, false, false, true>
+                     : rikfad_step_kernel<GT, false, false, false, true>;
+    return ragged ? step_kernel<GT, true>(reuse, shadow) : step_kernel<GT, false>(reuse, shadow);
+}
+
+StepKernel step_kernel(int grad_bytes, bool reuse, bool shadow, bool ragged, bool wide)
+{
+    return grad_bytes == 2 ? step_kernel<__nv_bfloat16>(reuse, shadow, ragged, wide)
+                           : step_kernel<float>(reuse, shadow, ragged, wide);
+}
+
+// Dynamic shared memory of the WIDE instantiations: the warps' column
+// accumulators and the widest band's C.
+constexpr int kWideSmemMax = sizeof(float) * (kWarps + 1) * kBandMax;
+
+size_t wide_smem(const Plan &p)
+{
+    return p.band_width == 0 ? 0 : sizeof(float) * (size_t)(kWarps + 1) * std::max(p.band_width, kPanelMax);
 }
 
 template <typename GT>
@@ -654,7 +672,7 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     int occ_min = 1 << 30;
     const int grad_bytes = grad_dtype == RIKFAD_GRAD_BF16 ? 2 : 4;
     for (const bool reuse : {true, false}) {        // the instantiations this handle launches
-        const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, has_ragged(shapes, ntensors));
+        const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, has_ragged(shapes, ntensors), false);
         RK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kThreads, 0),
                 "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         occ_min = std::min(occ_min, occ);
@@ -692,6 +710,27 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     h->shadow = shadow;
     h->ragged = has_ragged(shapes, ntensors);
     why = build_plan(shapes, ntensors, h->grad_bytes, h->max_blocks, h->plan, shadow);
+    h->wide_smem = wide_smem(h->plan);
+    if (why.empty() && h->wide_smem > 0 && !sweep) {
+        // The bands' instantiations, with the shared memory of this plan: allow
+        // it, and plan again if fewer of their blocks fit at once.
+        for (const bool reuse : {true, false}) {
+            const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, false, true);
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmemMax);
+            if (e == cudaSuccess)
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kThreads, h->wide_smem);
+            if (e != cudaSuccess || occ < 1) {
+                delete h;
+                return e != cudaSuccess ? cuda_fail(e, "step kernel with bands")
+                                        : fail(RIKFAD_ERR_CUDA, "step kernel cannot be resident on this device");
+            }
+            occ_min = std::min(occ_min, occ);
+        }
+        if (h->max_blocks != sms * occ_min) {
+            h->max_blocks = sms * occ_min;
+            why = build_plan(shapes, ntensors, h->grad_bytes, h->max_blocks, h->plan, shadow);
+        }
+    }
     if (!why.empty()) {
         delete h;
         return fail(RIKFAD_ERR_ARG, why);
@@ -889,6 +928,7 @@ RIKFAD_API int rikfad_step(rikfad_handle h, double step, float *const *x, const 
         a.decay = (float)decay_d;
         a.gain = (float)gain_d;
         a.eps = (float)h->hp.eps_stab;
+        a.band_width = std::max(h->plan.band_width, kPanelMax);
         a.guard = guard(h);
         a.chk = bounds(h);
         const bool reuse = (step == h->pending_step);
@@ -916,8 +956,8 @@ RIKFAD_API int rikfad_step(rikfad_handle h, double step, float *const *x, const 
                                    (int)h->plan.tile_groups.size() * kTileGroup, kThreads, s, a),
                         "launch rikfad_elements_kernel");
             else
-                RK_CUDA(launch_pdl(step_kernel(h->grad_bytes, reuse, h->shadow, h->ragged), h->plan.nblocks,
-                                   kThreads, s, a),
+                RK_CUDA(launch_pdl(step_kernel(h->grad_bytes, reuse, h->shadow, h->ragged, h->wide_smem > 0),
+                                   h->plan.nblocks, kThreads, s, a, h->wide_smem),
                         "launch rikfad_step_kernel");
         }
     }

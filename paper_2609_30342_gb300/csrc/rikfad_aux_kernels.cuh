@@ -68,7 +68,7 @@ __device__ __forceinline__ bool fin_item_ok(const FinParams &f, const FinItemDev
     if (f.resum_only)
         return true;
     const PanelDev pd = f.panels[it.panel];
-    const int ns = pd.slot_end - pd.slot_begin;
+    const int ns = panel_slots(pd);
     (void)ns;                  // read by the checks only
     return RK_DEV_CHECK(cb, pd.tensor == it.tensor && pd.col0 >= 0 &&
                                 (int64_t)pd.col0 + pd.width <= td.cols, kChkCols) &&
@@ -76,7 +76,8 @@ __device__ __forceinline__ bool fin_item_ok(const FinParams &f, const FinItemDev
            RK_DEV_CHECK(cb, pd.slot_begin >= 0 && ns >= 0 && pd.slot_end <= cb.nslots &&
                                 (it.chunk != 0 || ns <= kFinSplitSlots), kChkColpart) &&
            RK_DEV_CHECK(cb, ns == 0 || (f.slot_off[pd.slot_begin] >= 0 &&
-                                        f.slot_off[pd.slot_begin] + (int64_t)ns * pd.width <= cb.colpart_floats),
+                                        f.slot_off[pd.slot_begin] + (int64_t)(ns - 1) * pd.slot_stride +
+                                                pd.width <= cb.colpart_floats),
                         kChkColpart);
 }
 
@@ -141,18 +142,18 @@ __global__ void __launch_bounds__(kFinThreads) rikfad_finalize_kernel(FinParams 
             }
         }
     } else if (!f.resum_only && it.chunk == 0) {
-        // A panel's slots are consecutive in colpart, pd.width apart (the
-        // planner checks this), so every slot's load is issued at once and
+        // A panel's partials are pd.slot_stride apart in colpart (the planner
+        // checks this), so every slot's load is issued at once and
         // the sum is still taken in slot order.
         const PanelDev pd = f.panels[it.panel];
         const int64_t c = it.begin + threadIdx.x;
         if (c < it.end) {
-            const int ns = pd.slot_end - pd.slot_begin;
+            const int ns = panel_slots(pd);
             const float *cp = f.colpart + (ns > 0 ? f.slot_off[pd.slot_begin] : 0) + c;
             float v[kFinSplitSlots];
 #pragma unroll
             for (int u = 0; u < kFinSplitSlots; ++u)
-                v[u] = u < ns ? cp[(int64_t)u * pd.width] : 0.f;
+                v[u] = u < ns ? cp[(int64_t)u * pd.slot_stride] : 0.f;
             float acc = 0.f;
 #pragma unroll
             for (int u = 0; u < kFinSplitSlots; ++u)
@@ -171,8 +172,8 @@ __global__ void __launch_bounds__(kFinThreads) rikfad_finalize_kernel(FinParams 
         if (c < it.end) {
             const float *cp = f.colpart + f.slot_off[pd.slot_begin] + c;
 #pragma unroll 4
-            for (int s = warp; s < pd.slot_end - pd.slot_begin; s += kFinThreads / 32)
-                acc += cp[(int64_t)s * pd.width];
+            for (int s = warp, ns = panel_slots(pd); s < ns; s += kFinThreads / 32)
+                acc += cp[(int64_t)s * pd.slot_stride];
         }
         csum[warp][lane] = acc;
         __syncthreads();

@@ -103,6 +103,21 @@ __device__ __forceinline__ bool matrix_piece_ok(const CheckBounds &cb, const Pie
     return ok;
 }
 
+// A band led by piece q: its other panels follow as pieces of the same rows,
+// the band's columns end with the matrix and fit the launch's buffers, and its
+// partials lie side by side.
+__device__ __forceinline__ bool band_ok(const CheckBounds &cb, const PieceDev &pc, const TensorDev &td,
+                                        const PanelDev &pd, const PieceDev *pieces, int q, int q1, int band_width)
+{
+    (void)cb; (void)pc; (void)td; (void)pd; (void)pieces; (void)q; (void)q1; (void)band_width;
+    return RK_DEV_CHECK(cb, q + pc.band <= q1 && pc.panel + pc.band == td.panel0 + td.npanels, kChkPanel) &&
+           RK_DEV_CHECK(cb, pieces[q + pc.band - 1].band == 0 && pieces[q + pc.band - 1].begin == pc.begin &&
+                                pieces[q + pc.band - 1].end == pc.end, kChkRows) &&
+           RK_DEV_CHECK(cb, td.vec && pd.slot_step == pc.band && pd.slot_stride <= band_width &&
+                                (int64_t)pd.col0 + pd.slot_stride == td.cols, kChkCols) &&
+           RK_DEV_CHECK(cb, pc.colpart_off + pd.slot_stride <= cb.colpart_floats, kChkColpart);
+}
+
 __device__ __forceinline__ bool vector_piece_ok(const CheckBounds &cb, const PieceDev &pc,
                                                 const TensorDev &td, const void *x, const void *g,
                                                 const void *p, bool has_grad)

@@ -68,6 +68,7 @@ struct StepParams {
     float decay;               // e^{-alpha h}
     float gain;                // (1 - e^{-alpha h})/(mu alpha)
     float eps;                 // eps_stab
+    int band_width;            // WIDE: floats of a warp's column accumulators, columns of the widest band
     Guard guard;
     CheckBounds chk;           // read by checked builds only
 };
@@ -197,7 +198,8 @@ __device__ __forceinline__ float matrix_element(float &x, float p_hat, float g, 
 template <typename GT, bool REUSE, bool ACCUM = true, int RPW = 1>
 __device__ __forceinline__ void matrix_piece_vec(const StepParams &a, const PieceDev &pc,
                                                  const TensorDev &td, const PanelDev &pd,
-                                                 const float *Cs, float *red, float inv)
+                                                 const float *Cs, float *red, float inv,
+                                                 const int stride = kPanelMax)
 {
     constexpr int kRowLanes = 32 / RPW;                 // lanes per row
     constexpr int kRowChunk = kRowLanes * 8;            // columns per chunk of one row
@@ -212,7 +214,7 @@ __device__ __forceinline__ void matrix_piece_vec(const StepParams &a, const Piec
     float *P = a.pptr[pc.tensor];
     const float *R = a.fac + td.fac_off;
     float *rowpart = a.rowpart + td.rowpart_off + (int64_t)(pc.panel - td.panel0) * td.rows;
-    float *myred = red + warp * kPanelMax + half * (kPanelMax / RPW);
+    float *myred = red + warp * stride + half * (kPanelMax / RPW);
 
     for (int64_t r0 = pc.begin + kRowsPerWarp * warp; r0 < pc.end; r0 += kRowsPerWarp * kWarps) {
         const int64_t row = r0 + half;
@@ -280,6 +282,88 @@ __device__ __forceinline__ void matrix_piece_vec(const StepParams &a, const Piec
             racc = warp_sum(racc);
         }
         if (live && rl == 0)
+            rowpart[row] = racc;
+    }
+}
+
+// --------------------------------------------------------- matrix band
+//
+// Whole rows of a band (pd spans it), one row per warp, in 256-column chunks; a
+// last partial chunk of at most half a chunk is loaded together with the chunk
+// before it, so that it costs no round trip of its own.
+template <typename GT, bool REUSE>
+__device__ __forceinline__ void matrix_band(const StepParams &a, const PieceDev &pc, const TensorDev &td,
+                                            const PanelDev &pd, const float *Cs, float *red, float inv,
+                                            const int stride)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t n = td.cols;
+    const int w = pd.width, tail = w % kChunk;
+    const int w1 = tail <= kChunk / 2 ? w - tail - kChunk : w;      // columns before the joint pair
+    float *X = a.xptr[pc.tensor];
+    const GT *G = static_cast<const GT *>(a.gptr[pc.tensor]);
+    float *P = a.pptr[pc.tensor];
+    const float *R = a.fac + td.fac_off;
+    float *rowpart = a.rowpart + td.rowpart_off + (int64_t)(pc.panel - td.panel0) * td.rows;
+    float *myred = red + warp * stride;
+
+    for (int64_t row = pc.begin + warp; row < pc.end; row += kWarps) {
+        const float rhat = R[row] * inv;
+        const float a_cur = a.ex_cur * rhat;
+        const float a_prev = REUSE ? a_cur : a.ex_prev * rhat;
+        const int64_t base = row * n + pd.col0;
+        float racc = 0.f;
+        auto update = [&](int c, float (&xv)[8], float (&pv)[8], const Grad8<GT> &gv) {
+            const float4 c0 = *reinterpret_cast<const float4 *>(Cs + c);
+            const float4 c1 = *reinterpret_cast<const float4 *>(Cs + c + 4);
+            const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+            float q[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float e_cur = exp2f(a_cur * cv[e]);
+                const float e_prev = REUSE ? e_cur : exp2f(a_prev * cv[e]);
+                const float p1 = matrix_element(xv[e], pv[e], gv.get(e), e_cur, e_prev, a);
+                pv[e] = p1;
+                q[e] = p1 * p1;
+                racc += q[e];
+            }
+            store8(X + base + c, xv);
+            store8(P + base + c, pv);
+            float4 *r4 = reinterpret_cast<float4 *>(myred + c);
+            float4 s0 = r4[0], s1 = r4[1];
+            s0.x += q[0]; s0.y += q[1]; s0.z += q[2]; s0.w += q[3];
+            s1.x += q[4]; s1.y += q[5]; s1.z += q[6]; s1.w += q[7];
+            r4[0] = s0;
+            r4[1] = s1;
+        };
+        int c = lane * 8;
+#pragma unroll 1
+        for (; c < w1; c += kChunk) {
+            Grad8<GT> gv;
+            float xv[8], pv[8];
+            gv.load(G + base + c);
+            load8(X + base + c, xv);
+            load8(P + base + c, pv);
+            update(c, xv, pv, gv);
+        }
+        if (w1 < w) {
+            const int t = c + kChunk;
+            Grad8<GT> gv, gt;
+            float xv[8], pv[8], xt[8], pt[8];
+            gv.load(G + base + c);
+            load8(X + base + c, xv);
+            load8(P + base + c, pv);
+            if (t < w) {
+                gt.load(G + base + t);
+                load8(X + base + t, xt);
+                load8(P + base + t, pt);
+            }
+            update(c, xv, pv, gv);
+            if (t < w)
+                update(t, xt, pt, gt);
+        }
+        racc = warp_sum(racc);
+        if (lane == 0)
             rowpart[row] = racc;
     }
 }
@@ -543,7 +627,7 @@ __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const Pie
 // red[wi * kPanelMax + h * kPanelMax / RPW + c]; added warp by warp, groups in
 // order.
 template <int RPW>
-__device__ __forceinline__ void column_partials(const float *red, float *out, int w)
+__device__ __forceinline__ void column_partials(const float *red, float *out, int w, const int stride = kPanelMax)
 {
     for (int c = threadIdx.x; c < w; c += kThreads) {
         float s = 0.f;
@@ -551,7 +635,7 @@ __device__ __forceinline__ void column_partials(const float *red, float *out, in
         for (int wi = 0; wi < kWarps; ++wi)
 #pragma unroll
             for (int h = 0; h < RPW; ++h)
-                s += red[wi * kPanelMax + h * (kPanelMax / RPW) + c];
+                s += red[wi * stride + h * (kPanelMax / RPW) + c];
         out[c] = s;
     }
 }
@@ -574,11 +658,19 @@ struct RowsPerWarp {
     static constexpr int value = N;
 };
 
-template <typename GT, bool REUSE, bool SHADOW = false, bool RAGGED = false>
+// WIDE: the instantiation for handles with bands, whose column accumulators lie
+// in dynamic shared memory (40 M elements, bf16, panels / bands: width 1032 147 /
+// 129 us, 1376 145 / 125, 1800 249 / 132, 2600 150 / 129, 9000 147 / 129; taking the
+// rows' partial chunks 2 or 4 rows at a time after them instead: 130 to 143).
+template <typename GT, bool REUSE, bool SHADOW = false, bool RAGGED = false, bool WIDE = false>
 __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_kernel(StepParams a)
 {
-    __shared__ __align__(16) float Cs[kPanelMax];
-    __shared__ __align__(16) float red[kWarps * kPanelMax];
+    extern __shared__ __align__(16) float wide[];
+    __shared__ __align__(16) float Cs_[WIDE ? 4 : kPanelMax];
+    __shared__ __align__(16) float red_[WIDE ? 4 : kWarps * kPanelMax];
+    float *red = WIDE ? wide : red_;
+    const int stride = WIDE ? a.band_width : kPanelMax;
+    float *Cs = WIDE ? wide + kWarps * stride : Cs_;
     const int b = blockIdx.x;
     if (!RK_DEV_CHECK(a.chk, b < a.chk.nblocks, kChkBlock))
         return;
@@ -600,21 +692,40 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
         }
         if (!piece_panel_ok(a.chk, pc, td))
             continue;
-        const PanelDev pd = a.panels[pc.panel];
+        if (WIDE && pc.band == 0)
+            continue;                           // walked with an earlier panel
+        PanelDev pd = a.panels[pc.panel];
         // Block-uniform: every thread evaluates the same checks on the same
         // entries, so a skipped piece is skipped by the whole block.
         if (!matrix_piece_ok(a.chk, pc, td, pd, a.xptr[pc.tensor], a.gptr[pc.tensor], a.pptr[pc.tensor],
                              true))
             continue;
+        if (WIDE && pc.band > 1) {              // pd spans the band
+            if (!band_ok(a.chk, pc, td, pd, a.pieces, q, q1, a.band_width))
+                continue;
+            pd.width = pd.slot_stride;
+        }
         const int w = pd.width;
         // Stage this panel's C, clear the column accumulators.
         const float *C = a.fac + td.fac_off + td.rows + pd.col0;
         for (int c = threadIdx.x; c < w; c += kThreads)
             Cs[c] = C[c];
-        for (int i = threadIdx.x; i < kWarps * kPanelMax; i += kThreads)
-            red[i] = 0.f;
+        if (WIDE) {
+            for (int i = threadIdx.x; i < kWarps * stride / 4; i += kThreads)
+                reinterpret_cast<float4 *>(red)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+            for (int i = threadIdx.x; i < kWarps * kPanelMax; i += kThreads)
+                red[i] = 0.f;
+        }
         const float inv = inv_denominator(row_total(a.spart, td), a.eps);
         __syncthreads();
+        if (WIDE && pc.band > 1) {
+            matrix_band<GT, REUSE>(a, pc, td, pd, Cs, red, inv, stride);
+            __syncthreads();
+            column_partials<1>(red, a.colpart + pc.colpart_off, w, stride);
+            __syncthreads();
+            continue;
+        }
         // The RAGGED instantiations carry fewer row loops (1, 2 and 4 rows per
         // warp; 1 with SHADOW): with more of them the compiler spills inside the
         // loops (40 M elements, bf16, width 500: 182 us with all, 141 so; as
@@ -629,13 +740,13 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
                 else
                     matrix_piece_full<GT, false, N>(a, pc, td, pd, red);
             } else if (!RAGGED || td.vec) {
-                matrix_piece_vec<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv);
+                matrix_piece_vec<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv, stride);
             } else {
                 matrix_piece_ragged<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv);
             }
             __syncthreads();
             // Column partial sums of this piece, warps (and their lane groups) added in order.
-            column_partials<N>(red, a.colpart + pc.colpart_off, w);
+            column_partials<N>(red, a.colpart + pc.colpart_off, w, stride);
         };
         if ((SHADOW && RAGGED) || rpw == 1)
             piece(RowsPerWarp<1>());

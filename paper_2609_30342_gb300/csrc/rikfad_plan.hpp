@@ -66,9 +66,20 @@ struct PanelDev {
     int32_t col0;
     int32_t width;
     int32_t nch;          // ceil(width / kChunk)
-    int32_t slot_begin;   // column partial slots of this panel: [slot_begin, slot_end)
+    int32_t slot_begin;   // column partial slots of this panel: slot_begin, + slot_step, ..., below slot_end
     int32_t slot_end;
+    int32_t slot_step;    // 1, or the panels of its band
+    int32_t slot_stride;  // floats between consecutive partials: width, or the band's width
 };
+
+// Column partials of a panel.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int32_t panel_slots(const PanelDev &pd)
+{
+    return (pd.slot_end - pd.slot_begin + pd.slot_step - 1) / pd.slot_step;
+}
 
 // A tile is one small block's work in a pass that carries no sums from row to
 // row: up to tile_rows rows of a panel, or kTileElems elements of a vector.
@@ -93,7 +104,17 @@ struct PieceDev {
     int64_t begin;        // first row (matrix) or element (vector)
     int64_t end;
     int64_t colpart_off;  // matrix pieces: offset of the slot's width floats
+    int32_t band;         // panels walked together with this one, itself first (0: walked with an earlier one)
+    int32_t pad_;
 };
+
+// A band is a matrix's last panels, up to kBandMax columns together, where the
+// last is not a whole number of 256-column chunks: walked panel by panel, its
+// narrow panels stride over the rows in short segments and every row is visited
+// once per panel.  A block walks a band's rows whole, so the pieces of its panels
+// share their rows, their partials lie side by side, and the row sums go to the
+// first panel's row partials (the others' stay zero).
+constexpr int kBandMax = 2048;
 
 struct FinItemDev {
     int32_t kind;

@@ -21,6 +21,7 @@ struct Unit {
     int64_t cost;   // cost per row or element: its bytes, plus kRowCost for a matrix row
     int64_t gran;   // cut granularity
     int64_t bytes;  // compulsory bytes per row or element
+    int32_t band;   // matrix rows: panels walked together
 };
 
 }  // namespace
@@ -73,6 +74,13 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
         return "block budget must be >= 1";
     Plan p;
     std::vector<Unit> units;
+    // Bands are for the R-iKFAD instantiations without ragged rows.
+    const bool bands = !full_matrices && !has_ragged(shapes, ntensors);
+    double list_bytes = 0;
+    for (int t = 0; t < ntensors; ++t)
+        list_bytes += shapes[t].cols == 0 ? (double)shapes[t].rows * vector_elem_bytes(grad_bytes)
+                                          : (double)shapes[t].rows * shapes[t].cols * matrix_elem_bytes(grad_bytes);
+    const double share = std::max<double>(kMinBlockBytes, list_bytes / max_blocks);
 
     // Per-tensor layout: factor storage, column panels, row partials.
     int64_t fac = 0, rowpart = 0;
@@ -89,7 +97,7 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
             fac += round_up(td.rows, 8);
             if (td.rows > 0)
                 units.push_back({kElements, t, -1, td.rows, vector_elem_bytes(grad_bytes),
-                                 kElemGranule, vector_elem_bytes(grad_bytes)});
+                                 kElemGranule, vector_elem_bytes(grad_bytes), 0});
         } else {
             td.vec = (td.cols % 8 == 0) ? 1 : 0;
             fac += round_up(td.rows + td.cols, 8);
@@ -134,6 +142,26 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
             np = (int64_t)widths.size();
             td.npanels = (int32_t)np;
             td.panel0 = (int32_t)p.panels.size();
+            // The band (see rikfad_plan.hpp): the longest suffix of the panels
+            // within kBandMax columns, at least two, where the last panel is not
+            // a whole number of chunks and a share has rows enough for its longer
+            // rows (a warp takes whole ones): from 8 where the last panel is at
+            // most 32 columns, 96 where its rows per warp fill the lanes, else 32.
+            // us a step on one matrix, bf16, panels / bands: width 1800, 7 rows a
+            // share 28.3 / 24.4, 29 rows 99.0 / 60.2; 1376, 19 rows 34.9 / 35.8, 38
+            // rows 62.6 / 57.8, 96 rows 144.5 / 124.9; 1600, 33 rows 56.7 / 60.0, 82
+            // rows 126.9 / 127.1; the GPT2-XL-shaped list 4584 / 4524.
+            int64_t band0 = np, band_cols = 0;
+            if (bands && td.vec && np > 1 && widths[np - 1] % kChunk != 0) {
+                while (band0 > 0 && band_cols + widths[band0 - 1] <= kBandMax)
+                    band_cols += widths[--band0];
+                const int64_t last = widths[np - 1];
+                const int need = last <= kChunk / 8 ? 8 : last % (kChunk / 4) == 0 ? 96 : 32;
+                if (share < (double)need * band_cols * matrix_elem_bytes(grad_bytes))
+                    band0 = np;
+                else if (td.rows > 0)
+                    p.band_width = std::max(p.band_width, (int)band_cols);
+            }
             int64_t col0 = 0;
             for (int64_t k = 0; k < np; ++k) {
                 PanelDev pd{};
@@ -143,11 +171,14 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
                 col0 += widths[k];
                 pd.nch = (int32_t)ceil_div(pd.width, kChunk);
                 pd.slot_begin = pd.slot_end = 0;
-                if (td.rows > 0) {
-                    const int64_t b = pd.width * (full_matrices ? vector_elem_bytes(grad_bytes)
-                                                                : matrix_elem_bytes(grad_bytes));
+                pd.slot_step = k < band0 ? 1 : (int32_t)(np - band0);
+                pd.slot_stride = k < band0 ? pd.width : (int32_t)band_cols;
+                if (td.rows > 0 && k <= band0) {
+                    const int64_t w = k < band0 ? pd.width : band_cols;
+                    const int64_t b = w * (full_matrices ? vector_elem_bytes(grad_bytes) : matrix_elem_bytes(grad_bytes));
                     const int64_t c = td.vec ? b : b * kRaggedNum / kRaggedDen;
-                    units.push_back({kMatrixRows, t, (int32_t)p.panels.size(), td.rows, c + kRowCost, 1, b});
+                    units.push_back({kMatrixRows, t, (int32_t)p.panels.size(), td.rows, c + kRowCost, 1, b,
+                                     k < band0 ? 1 : (int32_t)(np - band0)});
                 }
                 p.panels.push_back(pd);
             }
@@ -193,26 +224,29 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
                     take = round_up(take, u.gran);
                     take = std::min(take, u.len - pos);
                 }
-                PieceDev pc{};
-                pc.kind = u.kind;
-                pc.tensor = u.tensor;
-                pc.panel = u.panel;
-                pc.begin = pos;
-                pc.end = pos + take;
-                pc.slot = -1;
-                pc.colpart_off = 0;
-                if (u.kind == kMatrixRows) {
-                    PanelDev &pd = p.panels[u.panel];
-                    const int32_t slot = (int32_t)p.slot_off.size();
-                    if (pd.slot_end == pd.slot_begin)
-                        pd.slot_begin = slot;
-                    pd.slot_end = slot + 1;
-                    pc.slot = slot;
-                    pc.colpart_off = colpart;
-                    p.slot_off.push_back(colpart);
-                    colpart += pd.width;
+                for (int32_t k = 0; k < std::max(u.band, 1); ++k) {
+                    PieceDev pc{};
+                    pc.kind = u.kind;
+                    pc.tensor = u.tensor;
+                    pc.panel = u.panel < 0 ? -1 : u.panel + k;
+                    pc.begin = pos;
+                    pc.end = pos + take;
+                    pc.slot = -1;
+                    pc.colpart_off = 0;
+                    pc.band = k == 0 ? u.band : 0;
+                    if (u.kind == kMatrixRows) {
+                        PanelDev &pd = p.panels[pc.panel];
+                        const int32_t slot = (int32_t)p.slot_off.size();
+                        if (pd.slot_end == pd.slot_begin)
+                            pd.slot_begin = slot;
+                        pd.slot_end = slot + 1;
+                        pc.slot = slot;
+                        pc.colpart_off = colpart;
+                        p.slot_off.push_back(colpart);
+                        colpart += pd.width;
+                    }
+                    p.pieces.push_back(pc);
                 }
-                p.pieces.push_back(pc);
                 acc += take * u.cost;
                 pos += take;
                 while (acc >= bound && block < G - 1) {
@@ -227,12 +261,12 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
         p.colpart_floats = colpart;
     }
 
-    // The finalise kernel addresses a panel's slots from its first one: they
-    // must be consecutive and one panel width apart in colpart.
+    // The finalise kernel addresses a panel's slots from its first one, by
+    // their step and stride.
     for (const PanelDev &pd : p.panels)
-        for (int32_t s = pd.slot_begin; s < pd.slot_end; ++s)
-            if (p.slot_off[s] != p.slot_off[pd.slot_begin] + (int64_t)(s - pd.slot_begin) * pd.width)
-                return "internal: slots of a panel are not contiguous";
+        for (int32_t s = pd.slot_begin, u = 0; s < pd.slot_end; s += pd.slot_step, ++u)
+            if (p.slot_off[s] != p.slot_off[pd.slot_begin] + (int64_t)u * pd.slot_stride)
+                return "internal: slots of a panel are not evenly spaced";
 
     // Finalise work: R in chunks of kFinThreads rows (each also yields one
     // partial sum of R), C in chunks of kFinColChunk columns of each panel.
@@ -254,7 +288,7 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
             const PanelDev &pd = p.panels[td.panel0 + k];
             // Many slots: 32-column items whose 8 warps split the slots; few
             // slots: one thread per column, 256 columns per item.
-            const bool split = pd.slot_end - pd.slot_begin > kFinSplitSlots;
+            const bool split = panel_slots(pd) > kFinSplitSlots;
             const int64_t step = split ? kFinColChunk : kFinThreads;
             for (int64_t c0 = 0; c0 < pd.width; c0 += step) {
                 FinItemDev it{};

@@ -16,6 +16,7 @@ struct Plan {
     std::vector<int64_t> slot_off;      // colpart offset of every slot
     std::vector<FinItemDev> fin_items;
     std::vector<TileGroupDev> tile_groups;   // every tensor, in memory order
+    int band_width = 0;                 // columns of the widest band (0: no bands)
     bool elements_only = false;         // no matrix has rows: the step is a pass over tiles
     int64_t fac_floats = 0;             // factors + element-wise friction (padded)
     int64_t rowpart_floats = 0;

@@ -107,3 +107,29 @@ def test_narrow_panels_match_oracle(method, grad_bf16):
             seeded.step(g, h)
             _compare(run, seeded, 1e-5, "step%d " % (k + 1))
     run.close()
+
+
+@pytest.mark.parametrize("grad_bf16", [True, False])
+def test_bands_match_oracle(grad_bf16):
+    """Matrices whose last panels are walked together: partial chunks of 8, 24,
+    40 and 136 columns, a band that is the whole row and one that is its end,
+    beside panels of whole chunks; constant and changing step sizes, from the
+    GPU's own state at every step (1e-5, per-element bound beyond)."""
+    shapes = [(5000, 1800), (2500, 1048), (2000, 1928), (1500, 2600), (300, 768), (77, 40), (1000, 0)]
+    from paper_2609_30342_gb300 import rikfad
+    blocks = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    plan = rikfad.plan_query(shapes, "bf16" if grad_bf16 else "f32", blocks)
+    same = (plan[1:, [0, 1, 5, 6]] == plan[:-1, [0, 1, 5, 6]]).all(axis=1) & (plan[1:, 2] == 0)
+    assert set(plan[1:][same][:, 1]) == {0, 1, 2, 3}       # these matrices have bands
+    hp = HParams(alpha=0.3, mu=1e-3, gamma=0.05, eps_stab=1e-8)
+    inp = workloads.ModelInputs(shapes, seed=64, g_std=1e-2, grad_bf16=grad_bf16)
+    run = DeviceRun(shapes, hp, grad_bf16, inp.X, inp.P)
+    depths = {t: (64.0, 128.0) for t in range(len(shapes))}     # 30 rows a warp, 8 warps, up to 50 slots
+    for k, h in enumerate((0.1, 0.1, 0.05)):
+        seeded = Tracked.from_gpu(run, depths)
+        g = inp.grads(k)
+        run.set_grads(g)
+        run.step(h)
+        seeded.step(g, h, hp, run.factors())
+        seeded.check(run, 1e-5, "step%d" % (k + 1))
+    run.close()
