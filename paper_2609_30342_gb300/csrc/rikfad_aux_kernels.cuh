@@ -68,7 +68,7 @@ __device__ __forceinline__ bool fin_item_ok(const FinParams &f, const FinItemDev
     if (f.resum_only)
         return true;
     const PanelDev pd = f.panels[it.panel];
-    const int ns = panel_slots(pd);
+    const int ns = pd.nslots;
     (void)ns;                  // read by the checks only
     return RK_DEV_CHECK(cb, pd.tensor == it.tensor && pd.col0 >= 0 &&
                                 (int64_t)pd.col0 + pd.width <= td.cols, kChkCols) &&
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kFinThreads) rikfad_finalize_kernel(FinParams 
         const PanelDev pd = f.panels[it.panel];
         const int64_t c = it.begin + threadIdx.x;
         if (c < it.end) {
-            const int ns = panel_slots(pd);
+            const int ns = pd.nslots;
             const float *cp = f.colpart + (ns > 0 ? f.slot_off[pd.slot_begin] : 0) + c;
             float v[kFinSplitSlots];
 #pragma unroll
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kFinThreads) rikfad_finalize_kernel(FinParams 
         if (c < it.end) {
             const float *cp = f.colpart + f.slot_off[pd.slot_begin] + c;
 #pragma unroll 4
-            for (int s = warp, ns = panel_slots(pd); s < ns; s += kFinThreads / 32)
+            for (int s = warp; s < pd.nslots; s += kFinThreads / 32)
                 acc += cp[(int64_t)s * pd.slot_stride];
         }
         csum[warp][lane] = acc;

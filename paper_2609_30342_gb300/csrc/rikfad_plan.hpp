@@ -70,16 +70,9 @@ struct PanelDev {
     int32_t slot_end;
     int32_t slot_step;    // 1, or the panels of its band
     int32_t slot_stride;  // floats between consecutive partials: width, or the band's width
+    int32_t nslots;       // column partials
+    int32_t pad_;
 };
-
-// Column partials of a panel.
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline int32_t panel_slots(const PanelDev &pd)
-{
-    return (pd.slot_end - pd.slot_begin + pd.slot_step - 1) / pd.slot_step;
-}
 
 // A tile is one small block's work in a pass that carries no sums from row to
 // row: up to tile_rows rows of a panel, or kTileElems elements of a vector.

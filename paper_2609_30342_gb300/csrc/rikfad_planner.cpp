@@ -170,7 +170,7 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
                 pd.width = (int32_t)widths[k];
                 col0 += widths[k];
                 pd.nch = (int32_t)ceil_div(pd.width, kChunk);
-                pd.slot_begin = pd.slot_end = 0;
+                pd.slot_begin = pd.slot_end = pd.nslots = 0;
                 pd.slot_step = k < band0 ? 1 : (int32_t)(np - band0);
                 pd.slot_stride = k < band0 ? pd.width : (int32_t)band_cols;
                 if (td.rows > 0 && k <= band0) {
@@ -240,6 +240,7 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
                         if (pd.slot_end == pd.slot_begin)
                             pd.slot_begin = slot;
                         pd.slot_end = slot + 1;
+                        ++pd.nslots;
                         pc.slot = slot;
                         pc.colpart_off = colpart;
                         p.slot_off.push_back(colpart);
@@ -288,7 +289,7 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
             const PanelDev &pd = p.panels[td.panel0 + k];
             // Many slots: 32-column items whose 8 warps split the slots; few
             // slots: one thread per column, 256 columns per item.
-            const bool split = panel_slots(pd) > kFinSplitSlots;
+            const bool split = pd.nslots > kFinSplitSlots;
             const int64_t step = split ? kFinColChunk : kFinThreads;
             for (int64_t c0 = 0; c0 < pd.width; c0 += step) {
                 FinItemDev it{};
