@@ -25,7 +25,7 @@
 // through the sums, the reciprocal and the exponential to the next kick, so a
 // step is one straight run of code: the loads and FMAs of the next gradient are
 // issued into that chain's gaps, and records and the end are looked at between
-// runs of steps.  119 ns a step for 4 x 3 and 187 for 6 x 5 (193 and 224 with
+// runs of steps.  119 ns a step for 4 x 3 and 164 for 6 x 5 (193 and 224 with
 // the gradient after the chain, a test for each step and a butterfly of four
 // levels for 4 x 3).  Large batches take the kernel further down, with one lane
 // per row or column.
@@ -260,7 +260,11 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) rikfad_quadratic_kerne
     const int steps = (int)(q.k1 - q.k0);
     int64_t ri = q.nrecord > 0 ? first_record_at_or_after(q.record, q.nrecord, q.k0) : 0;
     int next = record_in_launch(q, ri, steps);
-    float g, e2;
+    // The kick's bracket pb em - h g = e2 (pb o) + (pb f - h g): with the two
+    // products formed before e2 is there, two operations of the chain fewer (6 x 5
+    // 185 -> 164 ns a step, 2 x 2 102 -> 97; at 16 lanes 119 -> 122, not used).
+    constexpr bool kAhead = L != 16;
+    float g, e2, pbo = 0.f, pre = 0.f;
     // g = A vec(X) of the published x (four partial sums over every fourth
     // column, as two pairs advanced by paired FMAs) and e2 = expm1(-h/2 xi~) of
     // the current factors, for the step to come: one straight run of two
@@ -282,6 +286,10 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) rikfad_quadratic_kerne
         float g0, g1;
         unpack2(add2(g01, g23), g0, g1);
         g = g0 + g1;
+        if constexpr (kAhead) {
+            pbo = pb * o;
+            pre = fmaf(pb, f, -q.h * g);
+        }
         if (fabsf(z) > 0.0625f)
             e2 = expm1f(z);
     };
@@ -291,8 +299,8 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) rikfad_quadratic_kerne
         // between runs of steps.
         const int stop = next >= 0 ? next : steps;
         for (; s < stop; ++s) {
-            const float em = fmaf(e2, o, f);
-            pb = pb + fmaf(-q.h, g, pb * em);     // B (with the owed damping)
+            const float bracket = kAhead ? fmaf(e2, pbo, pre) : fmaf(-q.h, g, pb * fmaf(e2, o, f));
+            pb = pb + bracket;                    // B (with the owed damping)
             x = fmaf(q.h, pb, x);                 // A
             const float p1 = fmaf(pb, e2, pb);    // C, first half
             const float p1sq = p1 * p1;
@@ -710,10 +718,10 @@ extern "C" RIKFAD_API int rikfad_quadratic_run(int64_t batch, int64_t m, int64_t
     // warps are few per scheduler, one lane per row or column (fewer
     // instructions a system) beyond; later where that leaves a fifth or more of
     // the elements' slots empty.  ns a step, elements / lanes, measured at 16 |
-    // 1216 systems and throughput at 65536:  6 x 5  187 / 297 | 226 / 297, 6.9 /
+    // 1216 systems and throughput at 65536:  6 x 5  164 / 297 | 207 / 297, 6.9 /
     // 11.3 G system-steps/s;  4 x 3  119 / 143 | 120 / 143, 20 / 55;  3 x 7
-    // 176 / 183 | 205 / 184, 7.4 / 21;  2 x 2  102 / 101 | 103 / 101, 88 / 184;
-    // 10 x 3  175 / 258 | 229 / 319, 6.2 / 8.6.
+    // 168 / 183 | 197 / 184, 7.4 / 21;  2 x 2  97 / 101 | 99 / 101, 88 / 184;
+    // 10 x 3  163 / 258 | 214 / 319, 6.2 / 8.6.
     const int lanes = std::min(std::max(mb * nb, 4), 32);       // of the one-lane-per-element kernel
     const int64_t warps = (batch * lanes + 31) / 32;
     const int64_t slots = std::max(mb, nb) * std::min(m, n);    // of the one-lane-per-row kernel
