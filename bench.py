@@ -579,7 +579,8 @@ def run_ours(args, rank, world, local_rank):
         "hbm_gbs_step": round(alg_bytes / (ms_per_step / 1e3) / 1e9, 1),
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
                      "unit": "GB/s", "frac": round(achieved / peak, 4), "traffic": traffic,
-                     "kernel": "rikfad_step_kernel", "peak_source": peak_src,
+                     "kernel": "rikfad_elements_kernel" if args.method == "ikfad" else "rikfad_step_kernel",
+                     "peak_source": peak_src,
                      "peak_nominal": NOMINAL_HBM_GBS,
                      "frac_nominal": round(achieved / NOMINAL_HBM_GBS, 4),
                      "algorithmic_bytes_per_launch": kern_bytes,

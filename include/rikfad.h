@@ -350,7 +350,7 @@ RIKFAD_API int64_t rikfad_plan_query(const rikfad_shape *shapes, int ntensors, i
  *                 (start them at zero)
  * The first call on each device looks up the array's device address (and
  * may load the library's device code onto that GPU); make that first call
- * before any stream capture.  A call enqueues three kernels on `stream` and
+ * before any stream capture.  A call enqueues two or three kernels on `stream` and
  * writes every partial sum before it reads it, so nothing in the array needs
  * to start at zero and calls in sequence are independent.  All calls share
  * the one array: calls whose work overlaps on the GPU (unordered streams)
