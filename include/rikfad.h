@@ -393,7 +393,8 @@ RIKFAD_API int rikfad_step_matrix_noalloc(int64_t rows, int64_t cols, double ste
  *                 E = 1/2 vec(X)^T A vec(X) + 1/2 |P|_F^2 of the state after
  *                 record[r] steps is written to energy[r * batch + s].  Other
  *                 entries are skipped and their energies left untouched; a
- *                 list out of order loses the entries after the first descent.
+ *                 list out of order loses the entries after its first descent,
+ *                 up to the end of the launch that meets it (S below).
  *   energy        device, nrecord x batch floats (written)
  * The call is asynchronous on `stream`.  It runs the steps in launches of S
  * steps from its start (S = 65536 for batch <= 32768, a smaller power of two

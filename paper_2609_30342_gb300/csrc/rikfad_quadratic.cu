@@ -63,10 +63,13 @@
 #include <string>
 
 #include "rikfad.h"
+#include "rikfad_records.hpp"
 
 namespace rikfad {
 int report_error(int code, const std::string &msg);
 }
+
+using namespace rikfad;
 
 namespace {
 
@@ -120,30 +123,6 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
     uint64_t r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
-}
-
-// First index r with record[r] >= k (record ascending).
-__device__ __forceinline__ int64_t first_record_at_or_after(const int64_t *record, int64_t nrecord, int64_t k)
-{
-    int64_t lo = 0, hi = nrecord;
-    while (lo < hi) {
-        const int64_t mid = lo + (hi - lo) / 2;
-        if (record[mid] < k)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-// Step index of record[r] relative to the launch start, or -1 when there is
-// none within this launch.
-__device__ __forceinline__ int record_in_launch(const QuadParams &q, int64_t r, int steps)
-{
-    if (r >= q.nrecord)
-        return -1;
-    const int64_t rel = q.record[r] - q.k0;
-    return rel <= steps ? (int)rel : -1;
 }
 
 // exp(z) - 1.  For |z| <= 1/16 the exponential series without its constant
@@ -259,7 +238,7 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) rikfad_quadratic_kerne
 
     const int steps = (int)(q.k1 - q.k0);
     int64_t ri = q.nrecord > 0 ? first_record_at_or_after(q.record, q.nrecord, q.k0) : 0;
-    int next = record_in_launch(q, ri, steps);
+    int next = record_in_launch(q.record, q.nrecord, ri, q.k0, 0, steps);
     // The kick's bracket pb em - h g = e2 (pb o) + (pb f - h g): with the two
     // products formed before e2 is there, two operations of the chain fewer (6 x 5
     // 185 -> 164 ns a step, 2 x 2 102 -> 97; at 16 lanes 119 -> 122, not used).
@@ -345,7 +324,7 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) rikfad_quadratic_kerne
             if (live && a == 0)
                 q.energy[ri * q.batch + sys] = e;
             ++ri;
-            next = record_in_launch(q, ri, steps);
+            next = record_in_launch(q.record, q.nrecord, ri, q.k0, s, steps);
         }
         if (s == steps)
             break;
@@ -509,7 +488,7 @@ __global__ void __launch_bounds__(kQThreads, QLanes<LN, EPL>::MB) rikfad_quadrat
 
     const int steps = (int)(q.k1 - q.k0);
     int64_t ri = q.nrecord > 0 ? first_record_at_or_after(q.record, q.nrecord, q.k0) : 0;
-    int next = record_in_launch(q, ri, steps);
+    int next = record_in_launch(q.record, q.nrecord, ri, q.k0, 0, steps);
     float g[EPL], e2[EPL];
     // g = A vec(X) of the published x and e2 = expm1(-h/2 xi~) of the current
     // factors, for the step to come.  One straight run of independent chains, so
@@ -600,7 +579,7 @@ __global__ void __launch_bounds__(kQThreads, QLanes<LN, EPL>::MB) rikfad_quadrat
             if (live && l == 0)
                 q.energy[ri * q.batch + sys] = en;
             ++ri;
-            next = record_in_launch(q, ri, steps);
+            next = record_in_launch(q.record, q.nrecord, ri, q.k0, s, steps);
         }
         if (s == steps)
             break;

@@ -291,3 +291,23 @@ def test_large_batches_match_oracle(m, n):
         assert np.all(Eg[:, same] == Eg[:, [s]])
         for k in "XPRC":
             assert np.all(got[k][same] == got[k][s]), (k, s)
+
+
+@pytest.mark.parametrize("batch", [3, 12163])
+@pytest.mark.parametrize("rec,kept", [([5, 3, 40], 1), ([0, 30, 30, 2, 61], 3), ([61, 0], 1)])
+def test_records_out_of_order(rec, kept, batch):
+    """A list out of order, on both kernels (one lane per element, one per row):
+    the entries before the first descent get the energies of a run whose list
+    holds them alone, those after it stay untouched, and the state is that of a
+    run without records."""
+    A, X, P = workloads.dense_quadratic_batch(3, 2, [1, 2, 3])
+    idx = np.arange(batch) % 3
+    hp = HParams(1.0, 1.0, 0.05, 0.1)
+    plain, some, full = (_gpu_state(A[idx], X[idx], P[idx]) for _ in range(3))
+    _run(plain, 61, [], hp)
+    want = _run(some, 61, rec[:kept], hp)
+    got = _run(full, 61, rec, hp)
+    assert np.array_equal(got[:kept], want) and not np.any(np.isnan(want))
+    assert np.all(np.isnan(got[kept:]))
+    for k in "XPRC":
+        assert torch.equal(full[k], plain[k])
