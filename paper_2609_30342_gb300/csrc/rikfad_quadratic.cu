@@ -58,6 +58,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <string>
@@ -137,6 +138,18 @@ __device__ __forceinline__ float expm1_series(float z)
 __device__ __forceinline__ float expm1_small(float z)
 {
     return fabsf(z) <= 0.0625f ? expm1_series(z) : expm1f(z);
+}
+
+// 1 / (1^T R + eps); 0 below the normal range (zero included, Theorem 3's
+// convention), where the quotient can overflow: there R_i C_j / (1^T R) <= 1^T R
+// is below any friction that a step can show, while an infinite factor turns the
+// rows whose R_i is zero, and the lanes past the system's last row or column, into
+// NaN.  The friction is formed as (R_i inv)(C_j h/2) for the same reason: R_i inv
+// <= 1, whereas R_i C_j leaves the float32 range for factors beyond 1e+-19 (late in
+// a damped run, or early in a diverging one).
+__device__ __forceinline__ float inv_friction_denominator(float den)
+{
+    return den >= FLT_MIN ? __fdividef(1.f, den) : 0.f;
 }
 
 template <int MB, int NB>
@@ -258,9 +271,8 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) rikfad_quadratic_kerne
             g01 = fma2(arow2[2 * b4], v.x, g01);
             g23 = fma2(arow2[2 * b4 + 1], v.y, g23);
         }
-        const float den = S + q.eps;
-        const float inv = den > 0.f ? __fdividef(1.f, den) : 0.f;
-        const float z = L <= 16 ? ((Ri * Cj) * q.half_h) * inv : ((Ri * inv) * Cj) * q.half_h;
+        const float inv = inv_friction_denominator(S + q.eps);
+        const float z = (Ri * inv) * (Cj * q.half_h);
         e2 = expm1_series(z);
         float g0, g1;
         unpack2(add2(g01, g23), g0, g1);
@@ -494,8 +506,7 @@ __global__ void __launch_bounds__(kQThreads, QLanes<LN, EPL>::MB) rikfad_quadrat
     // factors, for the step to come.  One straight run of independent chains, so
     // that the FMAs of g fill the latencies of the factors' chain.
     auto prepare_step = [&]() {
-        const float den = S + q.eps;
-        const float inv = den > 0.f ? __fdividef(1.f, den) : 0.f;
+        const float inv = inv_friction_denominator(S + q.eps);
         const float fh = (F * inv) * q.half_h;
         float zmax = 0.f;
 #pragma unroll

@@ -311,3 +311,36 @@ def test_records_out_of_order(rec, kept, batch):
     assert np.all(np.isnan(got[kept:]))
     for k in "XPRC":
         assert torch.equal(full[k], plain[k])
+
+
+@pytest.mark.parametrize("batch", [3, 12163])
+@pytest.mark.parametrize("m,n", [(1, 1), (2, 2), (4, 4), (8, 2), (3, 2), (6, 5)])
+def test_factors_outside_the_normal_range(m, n, batch):
+    """eps = 0 and factors (and a momentum to match) from the subnormals, where a
+    run with linear damping ends up, to 1e20, where R_i C_j overflows: the state
+    stays finite and follows the oracle at the bounds of this file.  A tiny system's
+    momentum moves by h g alone (its friction is below 1e-38); a huge factor's
+    friction wipes P within the first half-damp."""
+    A, X, P = workloads.dense_quadratic_batch(m, n, [1, 2, 3])
+    hp = HParams(1.0, 1.0, 0.05, 0.0)
+    rng = np.random.default_rng(5)
+    unit_R, unit_C = rng.uniform(0.5, 1.0, (3, m)), rng.uniform(0.5, 1.0, (3, n))
+    unit_R *= 1.0 / unit_R.sum(1, keepdims=True)
+    unit_C *= 1.0 / unit_C.sum(1, keepdims=True)
+    scale = np.array([1e-20, 1e-21, 1.0])
+    factor = np.array([1e-40, 2e-42, 1e20])
+    X, P = (a * scale[:, None, None] for a in (X, P))
+    R, C = ((u * factor[:, None]).astype(np.float32) for u in (unit_R, unit_C))
+    if m > 1:
+        R[0, 0] = 0.0
+    idx = np.arange(batch) % 3
+    st = _gpu_state(A[idx], X[idx], P[idx], R[idx], C[idx])
+    _run(st, 5, [], hp)
+    for s in range(3):
+        _, Xo, Po, _, _ = _oracle(A[s], np.float32(X[s]), np.float32(P[s]), 5, [], hp, R[s], C[s])
+        for k, ref in zip("XP", (Xo, Po)):
+            got = st[k][s].cpu().numpy().astype(np.float64)
+            assert np.all(np.isfinite(got))
+            compare(k, got, ref, S_RTOL, 1.0)
+        for k in "RC":
+            assert torch.all(torch.isfinite(st[k][s]))
