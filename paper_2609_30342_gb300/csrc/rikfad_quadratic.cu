@@ -149,7 +149,8 @@ __device__ __forceinline__ float expm1_small(float z)
 // a damped run, or early in a diverging one).
 __device__ __forceinline__ float inv_friction_denominator(float den)
 {
-    return den >= FLT_MIN ? __fdividef(1.f, den) : 0.f;
+    const float inv = __fdividef(1.f, den);
+    return den < FLT_MIN ? 0.f : inv;
 }
 
 template <int MB, int NB>

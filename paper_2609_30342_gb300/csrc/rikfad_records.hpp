@@ -33,9 +33,10 @@ RK_HOST_DEVICE int64_t first_record_at_or_after(const int64_t *record, int64_t n
 // passed would never come.
 RK_HOST_DEVICE int record_in_launch(const int64_t *record, int64_t nrecord, int64_t r, int64_t k0, int s, int steps)
 {
-    if (r >= nrecord || record[r] < k0 + s || record[r] > k0 + steps)
+    if (r >= nrecord)
         return -1;
-    return (int)(record[r] - k0);
+    const int64_t rel = record[r] - k0;
+    return (uint64_t)(rel - s) <= (uint64_t)(steps - s) ? (int)rel : -1;    // s <= rel <= steps
 }
 
 }  // namespace rikfad
