@@ -1155,8 +1155,6 @@ RIKFAD_API int rikfad_export_state(rikfad_handle h, void *dev_dst, void *stream)
     if (!enqueue) {
         RK_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
         RK_CUDA(cudaMemcpy(dev_dst, &hd, sizeof hd, cudaMemcpyHostToDevice), "cudaMemcpy image header");
-    } else {
-        RK_CUDA(cudaPeekAtLastError(), "earlier CUDA error");
     }
     if (h->plan.fac_floats > 0)
         RK_CUDA(cudaMemcpyAsync((char *)dev_dst + kImageHeader, h->d_fac, sizeof(float) * h->plan.fac_floats,

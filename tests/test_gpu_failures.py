@@ -99,3 +99,27 @@ def test_sweep_state_allocated_only_when_selected():
     a.close()
     b.close()
     assert rikfad.debug_live_allocations() == live0
+
+
+def test_state_can_be_exported_after_a_failed_create():
+    """A create that the device has no memory for (2.2 TB) leaves CUDA's record of
+    the failed allocation behind; the state of a handle that was there before is
+    still exported, and is what it was."""
+    shapes = [(64, 40), (5, 0)]
+    opt = rikfad.RIKFAD(shapes, 0.3, 1e-3, 0.1, 1e-8, "f32")
+    opt.set_factors(0, [0.25] * 64, [0.5] * 40)
+    imgs = [torch.zeros(opt.state_image_bytes(), dtype=torch.uint8, device="cuda") for _ in range(2)]
+    opt.export_state(imgs[0])
+    with pytest.raises(rikfad.RikfadError) as e:
+        rikfad.RIKFAD([(1 << 20, 1 << 19)], 0.3, 1e-3, 0.1, 1e-8, "f32", method="ikfad_shadow")
+    assert e.value.args and "out of memory" in str(e.value)
+    try:
+        opt.export_state(imgs[1])
+        torch.cuda.synchronize()
+        assert torch.equal(imgs[0], imgs[1])
+    finally:
+        try:
+            opt.read_denominators()     # reports the record once, which clears it
+        except rikfad.RikfadError:
+            pass
+        opt.close()
