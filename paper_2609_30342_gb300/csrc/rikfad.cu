@@ -749,12 +749,14 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     if (!rc) rc = upload(&h->d_block_piece, p.block_piece, ws);
     if (!rc) rc = upload(&h->d_slot_off, p.slot_off, ws);
     if (!rc) rc = upload(&h->d_fin, p.fin_items, ws);
-    if (!rc) rc = upload(&h->d_tile_groups, p.tile_groups, ws);
     size_t state = 0;
     if (!rc) rc = alloc_zero(&h->d_fac, p.fac_floats, state);
     if (!rc) rc = alloc_zero(&h->d_rowpart, p.rowpart_floats, ws);
     if (!rc) rc = alloc_zero(&h->d_colpart, p.colpart_floats, ws);
     if (!rc) rc = alloc_zero(&h->d_spart, p.spart_floats, ws);
+    if (!rc && !(why = build_tiles(h->plan)).empty())
+        rc = fail(RIKFAD_ERR_ARG, why);
+    if (!rc) rc = upload(&h->d_tile_groups, p.tile_groups, ws);
     if (!rc) rc = alloc_zero(&h->d_den, std::max(ntensors, 1), ws);
     if (!rc) {
         cudaError_t e = rk_malloc_host((void **)&h->h_den, sizeof(float) * std::max(ntensors, 1),

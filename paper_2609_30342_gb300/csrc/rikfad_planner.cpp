@@ -303,18 +303,33 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
             }
         }
     }
-    // Tiles, in memory order: rows before panels.
     p.elements_only = true;
-    for (int t = 0; t < ntensors; ++t) {
-        const TensorDev &td = p.tensors[t];
+    for (const TensorDev &td : p.tensors)
         p.elements_only &= td.cols == 0 || td.rows == 0;
-        const int64_t tiles = td.rows == 0 ? 0 : ceil_div(td.rows, td.tile_rows) * std::max(td.npanels, 1);
-        for (int64_t i = 0; i < tiles; i += kTileGroup)
-            p.tile_groups.push_back({t, 0, i});
-    }
-    if (p.tile_groups.size() > (size_t)std::numeric_limits<int32_t>::max() / kTileGroup)
-        return "too many elements";
     plan = std::move(p);
+    return "";
+}
+
+std::string build_tiles(Plan &plan)
+{
+    auto tiles_of = [](const TensorDev &td) {
+        return td.rows == 0 ? 0 : ceil_div(td.rows, td.tile_rows) * std::max(td.npanels, 1);
+    };
+    // A launch's blocks: 2^31 tiles of at least kTileElems elements, beyond any
+    // memory.  Counted before anything is built.
+    int64_t groups = 0;
+    for (const TensorDev &td : plan.tensors) {
+        groups += ceil_div(tiles_of(td), kTileGroup);
+        if (groups > std::numeric_limits<int32_t>::max() / kTileGroup)
+            return "too many elements";
+    }
+    plan.tile_groups.clear();
+    plan.tile_groups.reserve((size_t)groups);
+    for (int t = 0; t < (int)plan.tensors.size(); ++t) {
+        const int64_t tiles = tiles_of(plan.tensors[t]);
+        for (int64_t i = 0; i < tiles; i += kTileGroup)
+            plan.tile_groups.push_back({t, 0, i});
+    }
     return "";
 }
 

@@ -15,7 +15,7 @@ struct Plan {
     std::vector<int32_t> block_piece;   // block b owns pieces [block_piece[b], block_piece[b+1])
     std::vector<int64_t> slot_off;      // colpart offset of every slot
     std::vector<FinItemDev> fin_items;
-    std::vector<TileGroupDev> tile_groups;   // every tensor, in memory order
+    std::vector<TileGroupDev> tile_groups;   // every tensor, in memory order (build_tiles)
     int band_width = 0;                 // columns of the widest band (0: no bands)
     bool elements_only = false;         // no matrix has rows: the step is a pass over tiles
     int64_t fac_floats = 0;             // factors + element-wise friction (padded)
@@ -35,6 +35,12 @@ struct Plan {
 // Add the in-order schedule (units, reduction trees) to a plan built by
 // build_plan.  Matrices keep their order; vectors come last.
 void build_sweep(const rikfad_shape *shapes, int ntensors, Plan &plan);
+
+// Add the tiles of every tensor: rows before panels.  Their number grows with the
+// elements (the rest of a plan with blocks, rows and columns), so that only a handle
+// has them, once its factors are allocated, and a plan query none.  Returns "" or an
+// error message.
+std::string build_tiles(Plan &plan);
 
 // Validate the shape list; returns "" or an error message.
 std::string check_shapes(const rikfad_shape *shapes, int ntensors);

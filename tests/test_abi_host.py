@@ -119,6 +119,20 @@ def test_plan_covers_every_element_once(shapes, nblocks, grad):
         assert per_block.max() <= fair + 2 * largest_unit + 1, (per_block.max(), fair)
 
 
+def test_plan_query_of_many_elements():
+    """A plan's cost goes with its blocks, not with the elements: a vector of 2^45
+    elements (2^34 tiles, 34 GB of table if the query built it) beside a matrix is
+    planned at once, every element once."""
+    import time
+    t0 = time.perf_counter()
+    plan = rikfad.plan_query([(1 << 45, 0), (64, 1800)], "bf16", 304)
+    assert time.perf_counter() - t0 < 5.0
+    vec = plan[plan[:, 1] == 0]
+    assert vec[0, 5] == 0 and vec[-1, 6] == 1 << 45 and np.array_equal(vec[1:, 5], vec[:-1, 6])
+    rows = plan[(plan[:, 1] == 1) & (plan[:, 3] == 0)]
+    assert rows[0, 5] == 0 and rows[-1, 6] == 64
+
+
 def test_plan_rejects_bad_arguments():
     with pytest.raises(rikfad.RikfadError):
         rikfad.plan_query([(-1, 3)], "bf16", 10)
