@@ -709,28 +709,30 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     h->max_blocks = sms * occ_min;
     h->shadow = shadow;
     h->ragged = has_ragged(shapes, ntensors);
-    why = build_plan(shapes, ntensors, h->grad_bytes, h->max_blocks, h->plan, shadow);
-    h->wide_smem = wide_smem(h->plan);
-    if (why.empty() && h->wide_smem > 0 && !sweep) {
-        // The bands' instantiations, with the shared memory of this plan: allow
-        // it, and plan again if fewer of their blocks fit at once.
+    // The bands' instantiations run as many blocks at once as the shared memory of
+    // the plan's widest band leaves (the in-order schedule has none of them).
+    cudaError_t wide_err = cudaSuccess;
+    auto resident = [&](const Plan &plan) {
+        int fit = occ_min;
         for (const bool reuse : {true, false}) {
             const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, false, true);
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmemMax);
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kThreads, h->wide_smem);
-            if (e != cudaSuccess || occ < 1) {
-                delete h;
-                return e != cudaSuccess ? cuda_fail(e, "step kernel with bands")
-                                        : fail(RIKFAD_ERR_CUDA, "step kernel cannot be resident on this device");
-            }
-            occ_min = std::min(occ_min, occ);
+            if (wide_err == cudaSuccess)
+                wide_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmemMax);
+            if (wide_err == cudaSuccess)
+                wide_err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kThreads, wide_smem(plan));
+            if (wide_err == cudaSuccess && occ < 1)
+                wide_err = cudaErrorLaunchOutOfResources;
+            fit = wide_err == cudaSuccess ? std::min(fit, occ) : 0;
         }
-        if (h->max_blocks != sms * occ_min) {
-            h->max_blocks = sms * occ_min;
-            why = build_plan(shapes, ntensors, h->grad_bytes, h->max_blocks, h->plan, shadow);
-        }
+        return sms * fit;
+    };
+    why = sweep ? build_plan(shapes, ntensors, h->grad_bytes, h->max_blocks, h->plan, shadow)
+                : build_resident_plan(shapes, ntensors, h->grad_bytes, h->max_blocks, h->plan, shadow, resident);
+    if (wide_err != cudaSuccess) {
+        delete h;
+        return cuda_fail(wide_err, "step kernel with bands");
     }
+    h->wide_smem = wide_smem(h->plan);
     if (!why.empty()) {
         delete h;
         return fail(RIKFAD_ERR_ARG, why);

@@ -63,4 +63,27 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
 inline int64_t matrix_elem_bytes(int grad_bytes) { return grad_bytes + 16; }
 inline int64_t vector_elem_bytes(int grad_bytes) { return grad_bytes + 24; }
 
+// build_plan for as many blocks as a plan's own launch lets run at once:
+// `resident(plan)` returns that number for a plan with bands, whose launch takes
+// shared memory by its widest band (0: cannot run; the result is then an error).
+// A plan for fewer blocks has larger shares and can so have wider bands: the
+// plan returned is one that `resident` was asked about last.  max_blocks is
+// lowered to what was planned for.
+template <typename F>
+std::string build_resident_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes, int &max_blocks, Plan &plan,
+                                bool full_matrices, F resident)
+{
+    for (;;) {
+        const std::string err = build_plan(shapes, ntensors, grad_bytes, max_blocks, plan, full_matrices);
+        if (!err.empty() || plan.band_width == 0)
+            return err;
+        const int fit = resident(plan);
+        if (fit < 1)
+            return "step kernel cannot be resident on this device";
+        if (fit >= max_blocks)
+            return "";
+        max_blocks = fit;
+    }
+}
+
 }  // namespace rikfad
