@@ -797,7 +797,7 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
         if (!rc) rc = alloc_zero((float **)&h->d_diag_norms, 4 * kDiagMaxBlocks, ws);
         if (!rc) rc = alloc_zero((float **)&h->d_diag_upart, 2 * kDiagMaxBlocks, ws);
         if (!rc) rc = alloc_zero((float **)&h->d_diag_v2part, 4 * kDiagMaxColBlocks, ws);
-        if (!rc) rc = alloc_zero((float **)&h->d_diag_state, (int64_t)(sizeof(DiagState) / sizeof(float)), ws);
+        if (!rc) rc = alloc_zero((float **)&h->d_diag_state, 2 * (int64_t)(sizeof(DiagState) / sizeof(float)), ws);
         if (!rc) {
             cudaError_t e = rk_malloc_host((void **)&h->h_diag_state, sizeof(DiagState), cudaHostAllocMapped);
             if (e != cudaSuccess)
@@ -1315,7 +1315,6 @@ RIKFAD_API int rikfad_friction_diagnostics(rikfad_handle h, int t, int max_iters
     d.upart = h->d_diag_upart;
     d.npart = h->d_diag_norms;
     d.v2part = h->d_diag_v2part;
-    d.st = h->d_diag_state;
     d.host = h->h_diag_state_dev;
     // kDiagIters iterations are enqueued at once, then two more whenever the
     // host finds them not enough; kernels queued past convergence return at once.
@@ -1326,6 +1325,8 @@ RIKFAD_API int rikfad_friction_diagnostics(rikfad_handle h, int t, int max_iters
         const int64_t stop = std::min<int64_t>(max_iters, (int64_t)it + (it == 0 ? kDiagIters : 2));
         for (; it < stop; ++it) {
             d.parity = it & 1;
+            d.st = h->d_diag_state + d.parity;
+            d.st_next = h->d_diag_state + (d.parity ^ 1);
             d.last = it + 1 == stop;
             auto rows = it == 0 ? (vec ? rikfad_diag_rows_kernel<true, true> : rikfad_diag_rows_kernel<true, false>)
                                 : (vec ? rikfad_diag_rows_kernel<false, true> : rikfad_diag_rows_kernel<false, false>);

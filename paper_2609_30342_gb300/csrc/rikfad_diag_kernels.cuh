@@ -45,8 +45,10 @@ constexpr int64_t kDiagMaxPartials = 1 << 24;   // floats of row-block partials 
 inline int diag_col_threads(int nblk) { return nblk > 128 ? 1024 : 256; }
 constexpr int kDiagIters = 4;            // iterations enqueued before the host first looks
 
-// State of one power iteration, in device memory; the record the host reads
-// is a copy in mapped host memory.
+// State of one power iteration, in device memory, kept twice and used by turns:
+// an iteration's kernels read one and its column kernel writes the other, so that
+// no block of a launch reads what another block of it writes.  The record the host
+// reads is a copy in mapped host memory.
 struct DiagState {
     double sigma2;     // ||xi v||^2 / ||v||^2 of the current iterate
     double f2;         // ||xi||^2
@@ -74,7 +76,8 @@ struct DiagParams {
     double *upart;             // nblk: sums of u_i^2
     double *npart;             // 2 x nblk: sums of xi^2 and (xi - xi~)^2
     double *v2part;            // 2 x ncb: sums of v_j^2
-    DiagState *st;
+    DiagState *st;             // of this iteration
+    DiagState *st_next;        // of the next
     DiagState *host;           // mapped host memory
 };
 
@@ -395,7 +398,7 @@ __global__ void __launch_bounds__(kThreads, FIRST && VEC ? 2 : 3) rikfad_diag_ro
 // warp 0 the W warp sums; its squares go to the other half of v2part.
 // Block 0 forms the quotient and tests convergence: |sigma^2 - previous| <= tol
 // sigma^2 from the second iteration on, or max_iters, or nothing left to
-// iterate on.
+// iterate on.  Once it is done, the launches that follow hand that on.
 __global__ void __launch_bounds__(1024) rikfad_diag_cols_kernel(DiagParams d)
 {
     constexpr int kU = 8;
@@ -406,8 +409,11 @@ __global__ void __launch_bounds__(1024) rikfad_diag_cols_kernel(DiagParams d)
     const int64_t n = d.td.cols;
     wait_for_predecessor();
     allow_successor_launch();
-    if (d.st->done)
+    if (d.st->done) {           // every block of the launch
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            d.st_next->done = 1;
         return;
+    }
     const int it = d.st->it + 1;
     // Totals, each by one warp: ||u||^2, ||v||^2, and (block 0, first iteration) the norms.
     if (warp < 2 || (it == 1 && blockIdx.x == 0 && warp < 4)) {
@@ -468,7 +474,7 @@ __global__ void __launch_bounds__(1024) rikfad_diag_cols_kernel(DiagParams d)
         if (v2 > 0.0 && (u2 > 0.0 || it == 1))
             s.sigma2 = u2 / v2;
         s.done = !(u2 > 0.0) || it >= d.max_iters || (it > 1 && fabs(s.sigma2 - prev) <= d.tol * s.sigma2);
-        *d.st = s;
+        *d.st_next = s;
         if (s.done || d.last)
             *d.host = s;
     }

@@ -168,3 +168,18 @@ def test_diagnostics_at_the_edges_of_the_kernels(m, n):
     cut = run.opt.friction_diagnostics(0, max_iters=1)
     assert cut[5] == 1.0 and cut[3] <= s1 * (1 + 1e-9)
     run.close()
+
+
+def test_a_launch_does_not_read_the_state_that_it_writes(tmp_path):
+    """The column kernel's first block writes the iteration's state while later
+    blocks of the same launch have yet to start: they must not see it
+    (tests/diag_state_check.cu drives the two kernels directly)."""
+    import os
+    import subprocess
+    from paper_2609_30342_gb300 import build as pkg_build
+    exe = tmp_path / "diag_state_check"
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "diag_state_check.cu")
+    subprocess.run([pkg_build.nvcc()] + pkg_build.ARCH + ["-O3", "-std=c++17", "-I", pkg_build.INCLUDE, "-I",
+                                                          pkg_build.CSRC, src, "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert out.returncode == 0 and out.stdout.strip().endswith("OK"), out.stdout + out.stderr
