@@ -203,11 +203,60 @@ __global__ void __launch_bounds__(kFinThreads) rikfad_finalize_kernel(FinParams 
 // blocks per SM with a contiguous share each, one row per warp.  A narrow
 // matrix's tile is taken as a run of elements: 400000 x 64 in 37 us instead of
 // 156, 1000000 x 8 in 16 instead of 287; 64-column panels beside wide ones gain
-// from the order (eight layers of width 1600: 1394 -> 388 us).
+// from the order (eight layers of width 1600: 1394 -> 388 us).  A
+// narrow ragged matrix's too (a warp a row left a block walking its tile of many
+// rows alone: 300000 x 1 687 us, 600000 x 5 200; so 10 and 12), and a copy of
+// element-wise friction's momentum (one load in flight per lane: 29296 x 1024 127
+// us; so 39).
 __device__ __forceinline__ void canonical_copy(const float *S, float *D, int64_t n)
 {
     for (int64_t e = threadIdx.x; e < n; e += kThreads)
         D[e] = S[e];
+}
+
+// A panel's rows as a run of units (elements or float4), of which a thread takes
+// every 256th from (i0, j0) on.
+struct PanelWalk {
+    int w, di, dj, i0, j0;
+    __device__ __forceinline__ explicit PanelWalk(int width)
+        : w(width), di(kThreads / width), dj(kThreads % width), i0((int)threadIdx.x / width), j0((int)threadIdx.x % width)
+    {
+    }
+    __device__ __forceinline__ void next(int &i, int &j) const
+    {
+        i += di;
+        j += dj;
+        if (j >= w) {
+            j -= w;
+            ++i;
+        }
+    }
+};
+
+// Copy `rows` rows of w units, n units apart; a thread has kU loads in flight.
+template <int kU, typename T>
+__device__ __forceinline__ void canonical_copy_panel(const T *S, T *D, int64_t n, int w, int rows)
+{
+    const PanelWalk walk(w);
+    const int cnt = rows * w;
+    int i = walk.i0, j = walk.j0;
+#pragma unroll 1
+    for (int q0 = threadIdx.x; q0 < cnt; q0 += kThreads * kU) {
+        T v[kU];
+        int a = i, b = j;
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            if (q0 + kThreads * u < cnt)
+                v[u] = __ldcs(S + a * n + b);
+            walk.next(a, b);
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            if (q0 + kThreads * u < cnt)
+                __stcs(D + i * n + j, v[u]);
+            walk.next(i, j);
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kThreads, 4) rikfad_canonical_kernel(CanonParams c)
@@ -245,10 +294,14 @@ __global__ void __launch_bounds__(kThreads, 4) rikfad_canonical_kernel(CanonPara
     if (!matrix_piece_ok(c.chk, pc, td, pd, D, nullptr, S, false))
         return;
     if (td.full) {      // element-wise friction: P already holds P_{n+1}
-        if (S != D)
-            for (int64_t row = pc.begin + warp; row < pc.end; row += kWarps)
-                for (int j = lane; j < pd.width; j += 32)
-                    D[row * td.cols + pd.col0 + j] = S[row * td.cols + pd.col0 + j];
+        const float *s0 = S + pc.begin * td.cols + pd.col0;
+        float *d0 = D + pc.begin * td.cols + pd.col0;
+        const int rows = (int)(pc.end - pc.begin);
+        if (S != D && td.vec)
+            canonical_copy_panel<4>(reinterpret_cast<const float4 *>(s0), reinterpret_cast<float4 *>(d0), td.cols / 4,
+                                    pd.width / 4, rows);
+        else if (S != D)
+            canonical_copy_panel<8>(s0, d0, td.cols, pd.width, rows);
         return;
     }
     const float *C = c.fac + td.fac_off + td.rows + pd.col0;
@@ -266,8 +319,9 @@ __global__ void __launch_bounds__(kThreads, 4) rikfad_canonical_kernel(CanonPara
                 v[k] = __ldcs(s4 + lane + 32 * k);
     };
     // A narrow matrix (one panel): its tile is a run of elements, of which every
-    // lane takes its share whatever the rows' width.
+    // lane takes its share whatever the rows' width (run: single elements).
     const bool flat = td.vec && td.npanels == 1 && pd.width <= 128;
+    const bool run = !td.vec && td.cols <= kRaggedRun;
     const int n4 = (int)(pc.end - pc.begin) * w4;       // flat: float4 of the tile
     const float4 *t4 = reinterpret_cast<const float4 *>(S + pc.begin * td.cols);
     auto load_flat = [&](int q0) {
@@ -280,7 +334,7 @@ __global__ void __launch_bounds__(kThreads, 4) rikfad_canonical_kernel(CanonPara
     float r = 0.f;
     if (flat) {
         load_flat(warp * 32 * kV + lane);
-    } else if (row < pc.end) {
+    } else if (!run && row < pc.end) {
         if (td.vec)
             load_row(row);
         r = R[row];
@@ -306,6 +360,36 @@ __global__ void __launch_bounds__(kThreads, 4) rikfad_canonical_kernel(CanonPara
                     v[k].w = (v[k].w * exp2f(a_prev * Cs[j + 3])) * c.damp_prev;
                     __stcs(d4 + q, v[k]);
                 }
+            }
+        }
+        return;
+    }
+    if (run) {
+        // A narrow ragged matrix: a run of elements too, of which a thread takes
+        // every 256th, 8 of them loaded before the first in-place store.
+        constexpr int kU = 8;
+        const int cnt = (int)(pc.end - pc.begin) * pd.width;
+        const float *s0 = S + pc.begin * td.cols;
+        float *d0 = D + pc.begin * td.cols;
+        const PanelWalk walk(pd.width);
+        int i = walk.i0, j = walk.j0;
+#pragma unroll 1
+        for (int q0 = threadIdx.x; q0 < cnt; q0 += kThreads * kU) {
+            float u8[kU], r8[kU];
+            int a = i, b = j;
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                if (q0 + kThreads * u < cnt) {
+                    u8[u] = __ldcs(s0 + q0 + kThreads * u);
+                    r8[u] = R[pc.begin + a];
+                }
+                walk.next(a, b);
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                if (q0 + kThreads * u < cnt)
+                    __stcs(d0 + q0 + kThreads * u, (u8[u] * exp2f((c.ex_prev * (r8[u] * inv)) * Cs[j])) * c.damp_prev);
+                walk.next(i, j);
             }
         }
         return;

@@ -25,6 +25,10 @@ constexpr int kFinThreads = 256;     // threads of the finalise kernel (= rows p
 constexpr int kFinColChunk = 32;     // columns per split column item (8 warps share its slots)
 constexpr int kFinSplitSlots = 8;    // panels with more slots than this get split column items
 constexpr int kTileElems = 2048;     // elements of a tile (8 per thread of a block)
+// Ragged matrices up to here have tiles that are runs of elements in the canonical
+// momentum's pass (a warp a row fills 256 columns a pass: 30 M elements of width 129
+// 93 us so and 74 as a run, 255 61 and 75).
+constexpr int kRaggedRun = 192;
 constexpr int kElemGranule = 8;      // element pieces start on multiples of 8 elements
 constexpr int64_t kMinBlockBytes = 64 * 1024;   // smallest share worth a block
 // The planner balances blocks on time, not bytes alone: each row of a matrix

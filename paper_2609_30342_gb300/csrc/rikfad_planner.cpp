@@ -136,9 +136,17 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
             // few elements spends its time on staging C).  Canonical momentum,
             // 16 / 32 rows a tile: GPT2-S 147.0 / 149.3 us, GPT2-Nano-shaped
             // 45.6 / 43.7, eight layers of width 1600 405 / 388.
-            td.tile_rows = widths.back() > kPanelMax / 2
-                               ? 2 * kWarps
-                               : 4 * kWarps * std::max<int64_t>(1, kTileElems / (kWarps * widths[0]));
+            // A narrow ragged matrix's tile is a run of elements: 2 kTileElems of them, 4
+            // where that still gives every block slot of the GPU (608) two tiles.  A wide
+            // ragged one's small tiles are for small matrices, whose tiles run at once
+            // (29 x 1025 11.3 us with 32 rows, 9.6 with 16; 100000 x 300 72.3 / 78.1).
+            const bool large = td.rows * td.cols >= (int64_t)2 * 608 * 4 * kTileElems;
+            if (!td.vec && td.cols <= kRaggedRun)
+                td.tile_rows = (large ? 4 : 2) * kTileElems / td.cols;
+            else if (widths.back() > kPanelMax / 2 || (!td.vec && !large))
+                td.tile_rows = 2 * kWarps;
+            else
+                td.tile_rows = 4 * kWarps * std::max<int64_t>(1, kTileElems / (kWarps * widths[0]));
             np = (int64_t)widths.size();
             td.npanels = (int32_t)np;
             td.panel0 = (int32_t)p.panels.size();

@@ -63,3 +63,35 @@ def test_element_lists_at_tile_edges(grad_bf16):
         seeded.step(g, h, HP, run.factors())
         seeded.check(run, 1e-5, "step%d" % (k + 1))
     run.close()
+
+
+RAGGED_SHAPES = [(8193, 1), (8192, 1), (3, 1), (1639, 5), (1638, 5), (64, 129), (63, 129), (32, 255), (33, 257),
+                 (16, 513), (15, 1001), (16, 1025), (7, 2047), (40, 3001), (1, 1027), (4096, 1), (4097, 1), (819, 5), (820, 5), (10007, 1003)]
+
+
+@pytest.mark.parametrize("method", ["rikfad", "ikfad_shadow"])
+def test_ragged_canonical_momentum_at_tile_edges(method):
+    """Ragged widths on both sides of a block's 256 threads and of a panel, with
+    row counts around a tile of 4096 elements (8192 for the
+    last, of 10 M).  Rank-1 friction: against the
+    oracle, and in place bit for bit as out of place; element-wise friction (with
+    8-wide matrices beside): a copy of the stored momentum, bit for bit."""
+    shapes = RAGGED_SHAPES + ([(1023, 8), (65, 1032)] if method == "ikfad_shadow" else [])
+    inp = workloads.ModelInputs(shapes, seed=73, g_std=1e-2)
+    run = DeviceRun(shapes, HP, True, inp.X, inp.P, method=method)
+    for k, h in enumerate((0.1, 0.05)):
+        seeded = Tracked.from_gpu(run) if method == "rikfad" else None
+        g = inp.grads(k)
+        run.set_grads(g)
+        run.step(h)
+        if seeded:
+            seeded.step(g, h, HP, run.factors())
+            seeded.check(run, 1e-5, "step%d" % (k + 1))
+    out = [torch.full_like(p, float("nan")) for p in run.p]
+    run.opt.canonical_momentum(run.p, out)
+    if method == "rikfad":
+        run.opt.materialize(run.p)
+    torch.cuda.synchronize()
+    for p, o in zip(run.p, out):
+        assert torch.equal(p, o)
+    run.close()
