@@ -727,15 +727,15 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
             continue;
         }
         // The RAGGED instantiations carry fewer row loops (1, 2 and 4 rows per
-        // warp; 1 with SHADOW): with more of them the compiler spills inside the
-        // loops (40 M elements, bf16, width 500: 182 us with all, 141 so; as
-        // functions of their own 197).
-        const int rpw = SHADOW && RAGGED ? 1 : rows_per_warp(!RAGGED || td.vec, w);
+        // warp; with SHADOW 1, and 8 for ragged panels up to 64 columns): with more
+        // of them the compiler spills inside the loops (40 M elements, bf16, width
+        // 500: 182 us with all, 141 so; as functions of their own 197).
+        const int rpw = SHADOW && RAGGED ? (td.vec || w > 64 ? 1 : 8) : rows_per_warp(!RAGGED || td.vec, w);
         // One call of the piece's path for its rows per warp.
         auto piece = [&](auto n) {
             constexpr int N = decltype(n)::value;
             if (SHADOW) {
-                if (!RAGGED || td.vec)
+                if (!RAGGED || (N == 1 && td.vec))
                     matrix_piece_full<GT, true, N>(a, pc, td, pd, red);
                 else
                     matrix_piece_full<GT, false, N>(a, pc, td, pd, red);
@@ -748,8 +748,10 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
             // Column partial sums of this piece, warps (and their lane groups) added in order.
             column_partials<N>(red, a.colpart + pc.colpart_off, w, stride);
         };
-        if ((SHADOW && RAGGED) || rpw == 1)
+        if (rpw == 1)
             piece(RowsPerWarp<1>());
+        else if (SHADOW && RAGGED)
+            piece(RowsPerWarp<8>());
         else if (rpw == 2)
             piece(RowsPerWarp<2>());
         else if (RAGGED || rpw == 4)
