@@ -146,7 +146,7 @@ struct rikfad_handle_s {
     int ntensors = 0;
     int grad_bytes = 4;
     size_t wide_smem = 0;           // dynamic shared memory of a step with bands (0: none)
-    bool ragged = false;            // a matrix has rows that are not 8-aligned
+    RaggedKind ragged = kNoRagged;  // matrices with rows that are not 8-aligned
     rikfad_hparams hp{};
     Plan plan;
     int max_blocks = 1;
@@ -393,25 +393,28 @@ using StepKernel = void (*)(StepParams);
 
 // The step kernel's instantiation for a handle's matrices.  Full-friction
 // matrices (shadow) have no pending factor, so reuse never applies to them.
-// `wide`: the list has bands (never with shadow or ragged).
-template <typename GT, bool RAGGED>
-StepKernel step_kernel(bool reuse, bool shadow)
+// `wide`: the list has bands (never with shadow or many ragged rows).
+template <typename GT, int RAGGED>
+StepKernel step_kernel(bool reuse, bool shadow, bool wide)
 {
     if (shadow)
         return rikfad_step_kernel<GT, false, true, RAGGED>;
+    if constexpr (RAGGED != kManyRagged)
+        if (wide)
+            return reuse ? rikfad_step_kernel<GT, true, false, RAGGED, true>
+                         : rikfad_step_kernel<GT, false, false, RAGGED, true>;
     return reuse ? rikfad_step_kernel<GT, true, false, RAGGED> : rikfad_step_kernel<GT, false, false, RAGGED>;
 }
 
 template <typename GT>
-StepKernel step_kernel(bool reuse, bool shadow, bool ragged, bool wide)
+StepKernel step_kernel(bool reuse, bool shadow, RaggedKind ragged, bool wide)
 {
-    if (wide)
-        return reuse ? rikfad_step_kernel<GT, true, false, false, true>
-                     : rikfad_step_kernel<GT, false, false, false, true>;
-    return ragged ? step_kernel<GT, true>(reuse, shadow) : step_kernel<GT, false>(reuse, shadow);
+    return ragged == kManyRagged  ? step_kernel<GT, kManyRagged>(reuse, shadow, wide)
+           : ragged == kFewRagged ? step_kernel<GT, kFewRagged>(reuse, shadow, wide)
+                                  : step_kernel<GT, kNoRagged>(reuse, shadow, wide);
 }
 
-StepKernel step_kernel(int grad_bytes, bool reuse, bool shadow, bool ragged, bool wide)
+StepKernel step_kernel(int grad_bytes, bool reuse, bool shadow, RaggedKind ragged, bool wide)
 {
     return grad_bytes == 2 ? step_kernel<__nv_bfloat16>(reuse, shadow, ragged, wide)
                            : step_kernel<float>(reuse, shadow, ragged, wide);
@@ -671,8 +674,9 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     // Persistent grid: as many blocks as can be resident at once.
     int occ_min = 1 << 30;
     const int grad_bytes = grad_dtype == RIKFAD_GRAD_BF16 ? 2 : 4;
+    const RaggedKind ragged = ragged_kind(shapes, ntensors);
     for (const bool reuse : {true, false}) {        // the instantiations this handle launches
-        const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, has_ragged(shapes, ntensors), false);
+        const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, ragged, false);
         RK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kThreads, 0),
                 "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         occ_min = std::min(occ_min, occ);
@@ -708,14 +712,14 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     h->shapes.assign(shapes, shapes + ntensors);
     h->max_blocks = sms * occ_min;
     h->shadow = shadow;
-    h->ragged = has_ragged(shapes, ntensors);
+    h->ragged = ragged;
     // The bands' instantiations run as many blocks at once as the shared memory of
     // the plan's widest band leaves (the in-order schedule has none of them).
     cudaError_t wide_err = cudaSuccess;
     auto resident = [&](const Plan &plan) {
         int fit = occ_min;
         for (const bool reuse : {true, false}) {
-            const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, false, true);
+            const void *k = (const void *)step_kernel(grad_bytes, reuse, shadow, ragged, true);
             if (wide_err == cudaSuccess)
                 wide_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmemMax);
             if (wide_err == cudaSuccess)

@@ -383,7 +383,8 @@ __device__ __forceinline__ void matrix_band(const StepParams &a, const PieceDev 
 template <typename GT, bool REUSE, bool ACCUM = true, int RPW = 1, int U = 8>
 __device__ __forceinline__ void matrix_piece_ragged(const StepParams &a, const PieceDev &pc,
                                                     const TensorDev &td, const PanelDev &pd,
-                                                    const float *Cs, float *red, float inv)
+                                                    const float *Cs, float *red, float inv,
+                                                    const int stride = kPanelMax)
 {
     constexpr int kRowLanes = 32 / RPW;                 // lanes per row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -395,7 +396,7 @@ __device__ __forceinline__ void matrix_piece_ragged(const StepParams &a, const P
     float *P = a.pptr[pc.tensor];
     const float *R = a.fac + td.fac_off;
     float *rowpart = a.rowpart + td.rowpart_off + (int64_t)(pc.panel - td.panel0) * td.rows;
-    float *myred = red + warp * kPanelMax + half * (kPanelMax / RPW);
+    float *myred = red + warp * stride + half * (kPanelMax / RPW);
 
     for (int64_t r0 = pc.begin + RPW * warp; r0 < pc.end; r0 += RPW * kWarps) {
         const int64_t row = r0 + half;
@@ -528,13 +529,13 @@ __device__ __forceinline__ float full_element(float &x, float &p, float &xi, flo
 // matrix_piece_ragged: one row per warp left most lanes of a narrow panel idle
 // (bf16 gradients, share of the 6.8 TB/s floor: width 24 0.20 -> 0.76, 64 0.49 ->
 // 0.88, 640 0.71 -> 0.87, 9000 0.39 -> 0.81).
-template <typename GT, bool VEC, int RPW>
+template <typename GT, bool VEC, int RPW, int U = 8>
 __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const PieceDev &pc,
                                                   const TensorDev &td, const PanelDev &pd,
                                                   float *red)
 {
     constexpr int kRowLanes = 32 / RPW;                 // lanes per row
-    constexpr int kU = 8;                               // ragged: elements per lane and pass
+    constexpr int kU = U;                               // ragged: elements per lane and pass
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rl = lane & (kRowLanes - 1), half = lane / kRowLanes;
     const int64_t n = td.cols;
@@ -662,7 +663,7 @@ struct RowsPerWarp {
 // in dynamic shared memory (40 M elements, bf16, panels / bands: width 1032 147 /
 // 129 us, 1376 145 / 125, 1800 249 / 132, 2600 150 / 129, 9000 147 / 129; taking the
 // rows' partial chunks 2 or 4 rows at a time after them instead: 130 to 143).
-template <typename GT, bool REUSE, bool SHADOW = false, bool RAGGED = false, bool WIDE = false>
+template <typename GT, bool REUSE, bool SHADOW = false, int RAGGED = kNoRagged, bool WIDE = false>
 __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_kernel(StepParams a)
 {
     extern __shared__ __align__(16) float wide[];
@@ -726,20 +727,31 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
             __syncthreads();
             continue;
         }
-        // The RAGGED instantiations carry fewer row loops (1, 2 and 4 rows per
+        if (RAGGED == kFewRagged && !td.vec) {  // one element per lane and load
+            if (SHADOW)
+                matrix_piece_full<GT, false, 1, 1>(a, pc, td, pd, red);
+            else
+                matrix_piece_ragged<GT, REUSE, true, 1, 1>(a, pc, td, pd, Cs, red, inv, stride);
+            __syncthreads();
+            column_partials<1>(red, a.colpart + pc.colpart_off, w, stride);
+            __syncthreads();
+            continue;
+        }
+        // The kManyRagged instantiations carry fewer row loops (1, 2 and 4 rows per
         // warp; with SHADOW 1, and 8 for ragged panels up to 64 columns): with more
         // of them the compiler spills inside the loops (40 M elements, bf16, width
         // 500: 182 us with all, 141 so; as functions of their own 197).
-        const int rpw = SHADOW && RAGGED ? (td.vec || w > 64 ? 1 : 8) : rows_per_warp(!RAGGED || td.vec, w);
+        constexpr bool kMany = RAGGED == kManyRagged;
+        const int rpw = SHADOW && kMany ? (td.vec || w > 64 ? 1 : 8) : rows_per_warp(!kMany || td.vec, w);
         // One call of the piece's path for its rows per warp.
         auto piece = [&](auto n) {
             constexpr int N = decltype(n)::value;
             if (SHADOW) {
-                if (!RAGGED || (N == 1 && td.vec))
+                if (!kMany || (N == 1 && td.vec))
                     matrix_piece_full<GT, true, N>(a, pc, td, pd, red);
                 else
                     matrix_piece_full<GT, false, N>(a, pc, td, pd, red);
-            } else if (!RAGGED || td.vec) {
+            } else if (!kMany || td.vec) {
                 matrix_piece_vec<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv, stride);
             } else {
                 matrix_piece_ragged<GT, REUSE, true, N>(a, pc, td, pd, Cs, red, inv);
@@ -750,11 +762,11 @@ __global__ void __launch_bounds__(kThreads, RIKFAD_STEP_MIN_BLOCKS) rikfad_step_
         };
         if (rpw == 1)
             piece(RowsPerWarp<1>());
-        else if (SHADOW && RAGGED)
+        else if (SHADOW && kMany)
             piece(RowsPerWarp<8>());
         else if (rpw == 2)
             piece(RowsPerWarp<2>());
-        else if (RAGGED || rpw == 4)
+        else if (kMany || rpw == 4)
             piece(RowsPerWarp<4>());
         else
             piece(RowsPerWarp<8>());

@@ -44,6 +44,15 @@ constexpr int64_t kRowCost = 256;
 // one ragged matrix finish last otherwise.  GPT2-S and one 1001 x 769 matrix
 // step in 412 us without the factor, 365 with it (363 with 3/2; the list alone 355).
 constexpr int64_t kRaggedNum = 5, kRaggedDen = 4;
+// How much of a list lies in matrices with ragged rows.  kFewRagged: so little (one
+// element in kFewRaggedShare at most) that they are moved one element per lane and
+// load, at kFewRaggedCost times the cost, in a step kernel that keeps the registers of
+// one without ragged rows: two of its blocks leave the finalise kernel's room on an
+// SM, those of a kManyRagged kernel do not.  us a step of the GPT2-Nano- and
+// GPT2-S-shaped lists with a 5 x 7 matrix, few / many: 99.8 / 104.2, 356 / 363;
+// eight layers of width 1600 938 / 992 (bands go with few).
+enum RaggedKind : int32_t { kNoRagged = 0, kFewRagged = 1, kManyRagged = 2 };
+constexpr int64_t kFewRaggedShare = 256, kFewRaggedCost = 8;
 
 enum PieceKind : int32_t { kMatrixRows = 0, kElements = 1 };
 enum FinKind : int32_t { kFinRows = 0, kFinCols = 1 };

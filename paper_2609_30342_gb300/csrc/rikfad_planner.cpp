@@ -54,12 +54,16 @@ std::string check_shapes(const rikfad_shape *shapes, int ntensors)
     return "";
 }
 
-bool has_ragged(const rikfad_shape *shapes, int ntensors)
+RaggedKind ragged_kind(const rikfad_shape *shapes, int ntensors)
 {
-    for (int t = 0; t < ntensors; ++t)
-        if (shapes[t].rows > 0 && shapes[t].cols % 8 != 0)
-            return true;
-    return false;
+    double ragged = 0, all = 0;
+    for (int t = 0; t < ntensors; ++t) {
+        const double e = (double)shapes[t].rows * std::max<int64_t>(shapes[t].cols, 1);
+        all += e;
+        if (shapes[t].cols % 8 != 0)
+            ragged += e;
+    }
+    return ragged == 0 ? kNoRagged : ragged * kFewRaggedShare <= all ? kFewRagged : kManyRagged;
 }
 
 std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes, int max_blocks,
@@ -74,8 +78,9 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
         return "block budget must be >= 1";
     Plan p;
     std::vector<Unit> units;
-    // Bands are for the R-iKFAD instantiations without ragged rows.
-    const bool bands = !full_matrices && !has_ragged(shapes, ntensors);
+    // Bands are for the R-iKFAD instantiations without many ragged rows.
+    const RaggedKind ragged = ragged_kind(shapes, ntensors);
+    const bool bands = !full_matrices && ragged != kManyRagged;
     double list_bytes = 0;
     for (int t = 0; t < ntensors; ++t)
         list_bytes += shapes[t].cols == 0 ? (double)shapes[t].rows * vector_elem_bytes(grad_bytes)
@@ -184,7 +189,7 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
                 if (td.rows > 0 && k <= band0) {
                     const int64_t w = k < band0 ? pd.width : band_cols;
                     const int64_t b = w * (full_matrices ? vector_elem_bytes(grad_bytes) : matrix_elem_bytes(grad_bytes));
-                    const int64_t c = td.vec ? b : b * kRaggedNum / kRaggedDen;
+                    const int64_t c = td.vec ? b : ragged == kFewRagged ? b * kFewRaggedCost : b * kRaggedNum / kRaggedDen;
                     units.push_back({kMatrixRows, t, (int32_t)p.panels.size(), td.rows, c + kRowCost, 1, b,
                                      k < band0 ? 1 : (int32_t)(np - band0)});
                 }

@@ -45,9 +45,9 @@ std::string build_tiles(Plan &plan);
 // Validate the shape list; returns "" or an error message.
 std::string check_shapes(const rikfad_shape *shapes, int ntensors);
 
-// Whether a matrix of the list has rows that are not 8-aligned (cols % 8 != 0),
-// which the step kernel updates in single elements.
-bool has_ragged(const rikfad_shape *shapes, int ntensors);
+// The ragged rows of a list (cols % 8 != 0), which the step kernel updates in
+// single elements.
+RaggedKind ragged_kind(const rikfad_shape *shapes, int ntensors);
 
 // Build the plan for at most max_blocks blocks.  grad_bytes is 2 or 4.
 // Returns "" on success or an error message.

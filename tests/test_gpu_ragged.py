@@ -133,3 +133,36 @@ def test_bands_match_oracle(grad_bf16):
         seeded.step(g, h, hp, run.factors())
         seeded.check(run, 1e-5, "step%d" % (k + 1))
     run.close()
+
+
+FEW = [(5, 7), (1, 1), (9, 33), (3, 1025), (70, 1), (17, 129), (2, 2051)]
+
+
+@pytest.mark.parametrize("method,base", [("rikfad", [(4000, 768), (33, 40), (1000, 0)]),
+                                         ("rikfad", [(5000, 1800), (300, 768), (1000, 0)]),
+                                         ("ikfad_shadow", [(4000, 768), (33, 40), (1000, 0)])])
+@pytest.mark.parametrize("grad_bf16", [True, False])
+def test_few_ragged_rows_match_oracle(method, base, grad_bf16):
+    """Lists that are 8-wide but for one element in 256 at most, without and with
+    bands: their ragged matrices (one panel and several, odd rows, buffers one
+    element on) and the others, from the GPU's own state at every step."""
+    shapes = base[:1] + FEW + base[1:]
+    ragged = sum(m * n for m, n in FEW)
+    assert ragged * 256 <= sum(workloads.numel(s) for s in shapes)
+    hp = SHADOW_HP if method == "ikfad_shadow" else HParams(alpha=0.3, mu=1e-3, gamma=0.05, eps_stab=1e-8)
+    inp = workloads.ModelInputs(shapes, seed=65, g_std=1e-2, grad_bf16=grad_bf16)
+    run = DeviceRun(shapes, hp, grad_bf16, inp.X, inp.P, method=method)
+    _off_by_one(run)
+    depths = {t: (64.0, 128.0) for t in range(len(shapes))}
+    for k, h in enumerate((0.1, 0.1, 0.05)):
+        g = inp.grads(k)
+        seeded = Tracked.from_gpu(run, depths) if method == "rikfad" else ShadowRef(shapes, *_gpu_state(run))
+        run.set_grads(g)
+        run.step(h)
+        if method == "rikfad":
+            seeded.step(g, h, hp, run.factors())
+            seeded.check(run, 1e-5, "step%d" % (k + 1))
+        else:
+            seeded.step(g, h)
+            _compare(run, seeded, 1e-5, "step%d " % (k + 1))
+    run.close()
