@@ -159,17 +159,22 @@ std::string build_plan(const rikfad_shape *shapes, int ntensors, int grad_bytes,
             // within kBandMax columns, at least two, where the last panel is not
             // a whole number of chunks and a share has rows enough for its longer
             // rows (a warp takes whole ones): from 8 where the last panel is at
-            // most 32 columns, 96 where its rows per warp fill the lanes, else 32.
+            // most 32 columns, 96 where its rows per warp fill the lanes, 68 where it is
+            // wider than half a panel and its last chunk nearly full (little is wasted
+            // without a band), else 32.
             // us a step on one matrix, bf16, panels / bands: width 1800, 7 rows a
             // share 28.3 / 24.4, 29 rows 99.0 / 60.2; 1376, 19 rows 34.9 / 35.8, 38
             // rows 62.6 / 57.8, 96 rows 144.5 / 124.9; 1600, 33 rows 56.7 / 60.0, 82
-            // rows 126.9 / 127.1; the GPT2-XL-shaped list 4584 / 4524.
+            // rows 126.9 / 127.1; 2040, 48 rows 99.2 / 102.6; 1528, 65 rows 99.1 / 101.0;
+            // 1440, 69 rows 103.0 / 101.7; the GPT2-XL-shaped list 4584 / 4524.
             int64_t band0 = np, band_cols = 0;
             if (bands && td.vec && np > 1 && widths[np - 1] % kChunk != 0) {
                 while (band0 > 0 && band_cols + widths[band0 - 1] <= kBandMax)
                     band_cols += widths[--band0];
                 const int64_t last = widths[np - 1];
-                const int need = last <= kChunk / 8 ? 8 : last % (kChunk / 4) == 0 ? 96 : 32;
+                const int need = last <= kChunk / 8         ? 8
+                                 : last % (kChunk / 4) == 0 ? 96
+                                 : last > kPanelMax / 2 && last % kChunk > kChunk * 5 / 8 ? 68 : 32;
                 if (share < (double)need * band_cols * matrix_elem_bytes(grad_bytes))
                     band0 = np;
                 else if (td.rows > 0)
