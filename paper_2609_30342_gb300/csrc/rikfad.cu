@@ -1322,7 +1322,6 @@ RIKFAD_API int rikfad_friction_diagnostics(rikfad_handle h, int t, int max_iters
     d.host = h->h_diag_state_dev;
     // kDiagIters iterations are enqueued at once, then two more whenever the
     // host finds them not enough; kernels queued past convergence return at once.
-    const bool vec = n % 4 == 0 && n <= kDiagStageCols;
     const size_t smem = n <= kDiagStageCols ? (size_t)((n + 3) / 4 * 8) * sizeof(float) : 0;
     const DiagState &st = *h->h_diag_state;
     for (int it = 0; it < max_iters;) {
@@ -1332,8 +1331,7 @@ RIKFAD_API int rikfad_friction_diagnostics(rikfad_handle h, int t, int max_iters
             d.st = h->d_diag_state + d.parity;
             d.st_next = h->d_diag_state + (d.parity ^ 1);
             d.last = it + 1 == stop;
-            auto rows = it == 0 ? (vec ? rikfad_diag_rows_kernel<true, true> : rikfad_diag_rows_kernel<true, false>)
-                                : (vec ? rikfad_diag_rows_kernel<false, true> : rikfad_diag_rows_kernel<false, false>);
+            auto rows = it == 0 ? diag_rows_kernel<true>(n) : diag_rows_kernel<false>(n);
             RK_CUDA(launch_pdl(rows, d.nblk, kThreads, s, d, smem), "launch rikfad_diag_rows_kernel");
             RK_CUDA(launch_pdl(rikfad_diag_cols_kernel, d.ncb, diag_col_threads(d.nblk), s, d), "launch rikfad_diag_cols_kernel");
         }

@@ -8,9 +8,11 @@
 // sigma_1 comes from power iteration on xi^T xi, on the device, two kernels an
 // iteration chained by programmatic dependent launch: the row kernel reads xi
 // once from memory (u = xi v, then this block's share of xi^T u from the rows
-// just read, still in L1 or L2), the column kernel adds the blocks' shares,
-// forms the next iterate and tests convergence.  The first row kernel also
-// takes the norms ||xi||^2 and ||xi - xi~||^2 from the same read.
+// just read, still in L1 or L2 up to kDiagStageCols columns; the rows that all
+// blocks of a wider one have in hand outgrow L2 from about 8000), the column
+// kernel adds the blocks' shares, forms the next iterate and tests convergence.
+// The first row kernel also takes the norms ||xi||^2 and ||xi - xi~||^2 from the
+// same read.
 //
 // The iterate's length does not matter: sigma^2 = ||xi v||^2 / ||v||^2 is formed
 // with the length of the float32 iterate itself, so no kernel waits for a norm
@@ -25,9 +27,10 @@
 //
 // Every reduction runs in a fixed order; float64 only adds per-row and
 // per-block partial sums.  Bound by launch and L2 latency for a layer's 2 to 10
-// MB, by the one read of xi for larger matrices.  Measured on GB300, six calls
-// for the layers of a GPT2-S block: 3800 to 7400 us (by seed) with four kernels an
-// iteration iteration in a captured graph and the plain quotient, 346 us so.
+// MB, by the reads of xi for larger matrices.  Measured on GB300, six calls for the
+// layers of a GPT2-S block: 3800 to 7400 us (by seed) with four kernels an
+// iteration in a captured graph and the plain quotient, 325 us so; 8192 x 8192 (268
+// MB) 453 us a call of 3 iterations, 4096 x 16384 647.
 #pragma once
 #include <algorithm>
 
@@ -142,10 +145,13 @@ __device__ __forceinline__ void add2(float &s, float &e, float s2, float e2)
 // time: wpr warps a row for u_i (columns interleaved between them), then every
 // thread its own columns for the block's share of xi^T u.  FIRST: the iterate
 // is C, scaled to at most unit length (all ones over sqrt(n) if C = 0), and the
-// norms are taken too.  VEC: 16-byte loads (n a multiple of 4, staged).
-template <bool FIRST, bool VEC>
-__global__ void __launch_bounds__(kThreads, FIRST && VEC ? 2 : 3) rikfad_diag_rows_kernel(DiagParams d)
+// norms are taken too.  WIDTH: 16-byte loads where n is a multiple of 4 (xi of
+// 4096 x 16384: 647 us a call with them, 926 without).
+enum DiagWidth { kDiagScalar, kDiagVec, kDiagVecStaged };
+template <bool FIRST, DiagWidth WIDTH>
+__global__ void __launch_bounds__(kThreads, FIRST && WIDTH != kDiagScalar ? 2 : 3) rikfad_diag_rows_kernel(DiagParams d)
 {
+    constexpr bool VEC = WIDTH != kDiagScalar;
     extern __shared__ __align__(16) float dsm[];
     __shared__ float2 ue[kWarps], nf[kWarps];
     __shared__ float us[kWarps];
@@ -156,7 +162,7 @@ __global__ void __launch_bounds__(kThreads, FIRST && VEC ? 2 : 3) rikfad_diag_ro
     allow_successor_launch();
     if (!FIRST && d.st->done)
         return;
-    const bool staged = n <= kDiagStageCols;
+    const bool staged = VEC ? WIDTH == kDiagVecStaged : n <= kDiagStageCols;
     float *wacc = staged ? dsm + (n + 3) / 4 * 4 : d.wpart + (int64_t)blockIdx.x * n;
     const float *v = staged ? dsm : FIRST ? d.C : d.v;
     float inv = 0.f, vscale = 1.f, vbias = 0.f;
@@ -244,7 +250,9 @@ __global__ void __launch_bounds__(kThreads, FIRST && VEC ? 2 : 3) rikfad_diag_ro
                     for (int k = 0; k < kU; ++k) {
                         const int q = q0 + k * step;
                         if (q < n4) {
-                            const float4 b = v4[q];
+                            const float4 b = FIRST && !staged ? make_float4(v_at(4 * q), v_at(4 * q + 1), v_at(4 * q + 2),
+                                                                            v_at(4 * q + 3))
+                                                              : v4[q];
                             dot2(sv.x, ev.x, xv[k].x, b.x);
                             dot2(sv.y, ev.y, xv[k].y, b.y);
                             dot2(sv.z, ev.z, xv[k].z, b.z);
@@ -390,6 +398,14 @@ __global__ void __launch_bounds__(kThreads, FIRST && VEC ? 2 : 3) rikfad_diag_ro
         else
             d.npart[2 * blockIdx.x + tid - 1] = t;
     }
+}
+
+template <bool FIRST>
+auto diag_rows_kernel(int64_t n)
+{
+    return n % 4 != 0             ? rikfad_diag_rows_kernel<FIRST, kDiagScalar>
+           : n <= kDiagStageCols ? rikfad_diag_rows_kernel<FIRST, kDiagVecStaged>
+                                 : rikfad_diag_rows_kernel<FIRST, kDiagVec>;
 }
 
 // Column kernel: cpb columns a block, 32 at a time.  The next iterate v =

@@ -54,9 +54,9 @@ int main()
         d.st = states + d.parity;
         d.st_next = states + (d.parity ^ 1);
         if (it == 0)
-            rikfad_diag_rows_kernel<true, false><<<d.nblk, kThreads>>>(d);
+            diag_rows_kernel<true>(n)<<<d.nblk, kThreads>>>(d);
         else
-            rikfad_diag_rows_kernel<false, false><<<d.nblk, kThreads>>>(d);
+            diag_rows_kernel<false>(n)<<<d.nblk, kThreads>>>(d);
         rikfad_diag_cols_kernel<<<d.ncb, diag_col_threads(d.nblk)>>>(d);
         if (cudaDeviceSynchronize() != cudaSuccess) {
             std::printf("FAIL %s\n", cudaGetErrorString(cudaGetLastError()));
