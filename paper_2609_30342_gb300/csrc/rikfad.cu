@@ -231,7 +231,7 @@ int upload(T **dst, const std::vector<T> &src, size_t &bytes)
     return RIKFAD_OK;
 }
 
-int alloc_zero(float **dst, int64_t floats, size_t &bytes)
+int alloc_floats(float **dst, int64_t floats, size_t &bytes)
 {
     *dst = nullptr;
     if (floats <= 0)
@@ -241,8 +241,20 @@ int alloc_zero(float **dst, int64_t floats, size_t &bytes)
     if (e != cudaSuccess)
         return alloc_fail(e, "cudaMalloc");
     bytes += nb;
-    RK_CUDA(cudaMemset(*dst, 0, nb), "cudaMemset");
     return RIKFAD_OK;
+}
+
+int set_zero(float *dst, int64_t floats)
+{
+    if (floats > 0)
+        RK_CUDA(cudaMemset(dst, 0, (size_t)floats * sizeof(float)), "cudaMemset");
+    return RIKFAD_OK;
+}
+
+int alloc_zero(float **dst, int64_t floats, size_t &bytes)
+{
+    const int rc = alloc_floats(dst, floats, bytes);
+    return rc ? rc : set_zero(*dst, floats);
 }
 
 int ptrtable_init(PtrTable &t, int count, size_t &bytes)
@@ -756,13 +768,14 @@ int create_impl(const rikfad_shape *shapes, int ntensors, const rikfad_hparams *
     if (!rc) rc = upload(&h->d_slot_off, p.slot_off, ws);
     if (!rc) rc = upload(&h->d_fin, p.fin_items, ws);
     size_t state = 0;
-    if (!rc) rc = alloc_zero(&h->d_fac, p.fac_floats, state);
-    if (!rc) rc = alloc_zero(&h->d_rowpart, p.rowpart_floats, ws);
-    if (!rc) rc = alloc_zero(&h->d_colpart, p.colpart_floats, ws);
-    if (!rc) rc = alloc_zero(&h->d_spart, p.spart_floats, ws);
+    if (!rc) rc = alloc_floats(&h->d_fac, p.fac_floats, state);
     if (!rc && !(why = build_tiles(h->plan)).empty())
         rc = fail(RIKFAD_ERR_ARG, why);
     if (!rc) rc = upload(&h->d_tile_groups, p.tile_groups, ws);
+    if (!rc) rc = set_zero(h->d_fac, p.fac_floats);     // after the uploads, which would wait for it
+    if (!rc) rc = alloc_zero(&h->d_rowpart, p.rowpart_floats, ws);
+    if (!rc) rc = alloc_zero(&h->d_colpart, p.colpart_floats, ws);
+    if (!rc) rc = alloc_zero(&h->d_spart, p.spart_floats, ws);
     if (!rc) rc = alloc_zero(&h->d_den, std::max(ntensors, 1), ws);
     if (!rc) {
         cudaError_t e = rk_malloc_host((void **)&h->h_den, sizeof(float) * std::max(ntensors, 1),
