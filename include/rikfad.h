@@ -402,7 +402,10 @@ RIKFAD_API int rikfad_step_matrix_noalloc(int64_t rows, int64_t cols, double ste
  * starts from the stored X, P, R, C.  A run split into consecutive calls at
  * a multiple of S (the second starting from the first's outputs, its record
  * indices counted from its own start) is therefore bit-identical to one
- * call; a split elsewhere agrees to float32 rounding.  Errors:
+ * call; a split elsewhere agrees to float32 rounding.  Large batches are mapped
+ * to the GPU otherwise than small ones: the same system agrees between batches
+ * of different sizes to float32 rounding, and bit for bit within one batch size.
+ * Errors:
  * RIKFAD_ERR_ARG for sizes or hyperparameters out of range or a NULL pointer
  * that is needed, RIKFAD_ERR_ALIGN for a pointer not aligned to its element
  * type, RIKFAD_ERR_CUDA for a launch failure; messages via rikfad_last_error.

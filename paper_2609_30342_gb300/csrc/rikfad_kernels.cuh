@@ -619,13 +619,8 @@ __device__ __forceinline__ void matrix_piece_full(const StepParams &a, const Pie
 #define RIKFAD_STEP_MIN_BLOCKS 2
 #endif
 
-// SHADOW: the instantiation for handles whose matrices all keep element-wise
-// friction with shadow factors (the R-iKFAD instantiations carry no code for
-// it, nor it any for them).  RAGGED: the instantiation for handles with a
-// matrix whose rows are not 8-aligned; the paths of such matrices take more
-// registers than the 8-wide ones, so other handles do not carry them.
 // out[c] = the piece's column sums: warp wi's lane group h holds its share at
-// red[wi * kPanelMax + h * kPanelMax / RPW + c]; added warp by warp, groups in
+// red[wi * stride + h * kPanelMax / RPW + c]; added warp by warp, groups in
 // order.
 template <int RPW>
 __device__ __forceinline__ void column_partials(const float *red, float *out, int w, const int stride = kPanelMax)
@@ -659,6 +654,13 @@ struct RowsPerWarp {
     static constexpr int value = N;
 };
 
+// SHADOW: the instantiation for handles whose matrices all keep element-wise
+// friction with shadow factors (the R-iKFAD instantiations carry no code for
+// it, nor it any for them).  RAGGED: how much of the list lies in matrices whose
+// rows are not 8-aligned (RaggedKind).  The batched loops of kManyRagged take 126 to
+// 128 registers, WIDE 118 to 122 and SHADOW 116, where the others take 103 to 109: two
+// blocks of up to 112 leave an SM the 8192 registers of a finalise block, which can
+// then wait beside them for the last one; beside the others it starts as they drain.
 // WIDE: the instantiation for handles with bands, whose column accumulators lie
 // in dynamic shared memory (40 M elements, bf16, panels / bands: width 1032 147 /
 // 129 us, 1376 145 / 125, 1800 249 / 132, 2600 150 / 129, 9000 147 / 129; taking the

@@ -25,7 +25,7 @@
 // through the sums, the reciprocal and the exponential to the next kick, so a
 // step is one straight run of code: the loads and FMAs of the next gradient are
 // issued into that chain's gaps, and records and the end are looked at between
-// runs of steps.  119 ns a step for 4 x 3 and 164 for 6 x 5 (193 and 224 with
+// runs of steps.  112 ns a step for 4 x 3 and 161 for 6 x 5 (193 and 224 with
 // the gradient after the chain, a test for each step and a butterfly of four
 // levels for 4 x 3).  Large batches take the kernel further down, with one lane
 // per row or column.
@@ -255,7 +255,9 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) rikfad_quadratic_kerne
     int next = record_in_launch(q.record, q.nrecord, ri, q.k0, 0, steps);
     // The kick's bracket pb em - h g = e2 (pb o) + (pb f - h g): with the two
     // products formed before e2 is there, two operations of the chain fewer (6 x 5
-    // 185 -> 164 ns a step, 2 x 2 102 -> 97; at 16 lanes 119 -> 122, not used).
+    // 185 -> 164 ns a step, 2 x 2 102 -> 97; at 16 lanes 119 -> 122, not used).  It
+    // rounds h g once more than the fused form; over 24 settings the error against
+    // 64 bits is that of the fused form to 0.2% in the mean, 3% for single ones.
     constexpr bool kAhead = L != 16;
     float g, e2, pbo = 0.f, pre = 0.f;
     // g = A vec(X) of the published x (four partial sums over every fourth
@@ -415,10 +417,11 @@ int pow2_ceil(int v)
 // lanes only (its total is the sum of the EPL results, so 1^T R needs no
 // butterfly of its own).  EPL rows of A per lane are held in registers (160 of
 // them for 6 x 5: 8 warps an SM).  Bound by the FP32 pipe (64% of its cycles for
-// 6 x 5: 16 paired FMAs per system and step, and ~30 operations per element)
-// and by latency between them; 70 warp instructions per 6 x 5 system and step
-// against 119 with a lane per element.  65536 systems of 6 x 5: 7.1 -> 11.3 G
-// system-steps/s.
+// 6 x 5: 80 paired FMAs per lane and step, for 4 systems a warp, and ~30
+// operations per element) and by latency between them; 70 warp instructions per
+// 6 x 5 system and step against 119 with a lane per element.  65536 systems of
+// 6 x 5: 7.4 -> 11.9 G system-steps/s.  With one row or column the lanes are the same
+// in number, and what is saved is the exchange of the squares through shared memory.
 template <int LN, int EPL>
 struct QLanes {
     static constexpr int D = LN * EPL < 32 ? LN * EPL : 32;      // largest d (m n <= 32)
@@ -708,11 +711,14 @@ extern "C" RIKFAD_API int rikfad_quadratic_run(int64_t batch, int64_t m, int64_t
     // One lane per element (more lanes a system: the shorter step) while its
     // warps are few per scheduler, one lane per row or column (fewer
     // instructions a system) beyond; later where that leaves a fifth or more of
-    // the elements' slots empty.  ns a step, elements / lanes, measured at 16 |
-    // 1216 systems and throughput at 65536:  6 x 5  164 / 297 | 207 / 297, 6.9 /
-    // 11.3 G system-steps/s;  4 x 3  119 / 143 | 120 / 143, 20 / 55;  3 x 7
-    // 168 / 183 | 197 / 184, 7.4 / 21;  2 x 2  97 / 101 | 99 / 101, 88 / 184;
-    // 10 x 3  163 / 258 | 214 / 319, 6.2 / 8.6.
+    // the elements' slots empty.  ns a step, elements / lanes, measured at 16
+    // systems | just beyond the line, and throughput in G system-steps/s at 65536:
+    //   6 x 5  161 / 271 | 255 / 275, 7.4 / 11.9     4 x 3  112 / 131 | 186 / 134, 20 / 57
+    //   3 x 7  159 / 174 | 242 / 176, 8.4 / 22       2 x 2  95 / 91 | 140 / 116, 106 / 189
+    //   10 x 3 158 / 222 | 280 / 307, 6.6 / 9.0      8 x 1  100 / 117 | 161 / 145, 50 / 66
+    //   16 x 1 116 / 134 | 214 / 175, 18 / 28        32 x 1 161 / 160 | 276 / 221, 7.1 / 10.1
+    // (6 x 5 and 10 x 3 at two warps per scheduler, where their line is three).  A
+    // system's low bits so depend on the batch that it is run in.
     const int lanes = std::min(std::max(mb * nb, 4), 32);       // of the one-lane-per-element kernel
     const int64_t warps = (batch * lanes + 31) / 32;
     const int64_t slots = std::max(mb, nb) * std::min(m, n);    // of the one-lane-per-row kernel
