@@ -760,7 +760,7 @@ def run_g0(args, rank, world, local_rank):
                    "parallelism": "replicas" if world > 1 else "single GPU"},
         "roofline": {"bound": "alu", "achieved": round(achieved, 3), "peak": round(FP32_PEAK_TFLOPS, 1),
                      "unit": "TFLOP/s", "frac": round(achieved / FP32_PEAK_TFLOPS, 4), "traffic": None,
-                     "kernel": "rikfad_quadratic_kernel<8,8>",
+                     "kernel": "rikfad_quadratic_lanes_kernel<8,5>",
                      "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz",
                      "flops_per_system_step": g0_flops(m, n)},
         "e2e": e2e,
